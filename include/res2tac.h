@@ -113,9 +113,11 @@ typedef struct res2tac_pair {
  * row_cost: costs of the row-path kernel: 1 = read from the cost volume, 2 = recomputed from the
  *   census descriptors inside the walk (popcount of the XOR per step; census cost with
  *   row_mode 2 and D = 32 agg_dpl only, other settings read the volume).
- * Automatic values: agg_dpl 2 for D <= 64, 4 for D <= 128, else 8; agg_warps 2; wta_chunk 128;
- * shear_dpl 16; row_mode 2; shear_cpl 2 at D = 128, else 1; cost_mode 1 (measured faster);
- * row_cost 1. */
+ * Automatic values: agg_dpl 2 for D <= 64, 4 for D <= 128, else 8; agg_warps 2; shear_dpl 16;
+ * row_mode 2; cost_mode 1 (measured faster); row_cost 1; wta_chunk 64 and shear_cpl 1 for a context
+ * on path planes (see res2tac_create), else wta_chunk 128 and shear_cpl 2 at D = 128, 1 otherwise.
+ * A context on path planes uses them for calls with shear_dpl 16, row_mode 2, cost_mode 1 and
+ * row_cost 1 (agg_warps has no effect there), and sums in place with any other setting. */
 typedef struct res2tac_tuning {
   int32_t agg_dpl;
   int32_t agg_warps;
@@ -130,6 +132,11 @@ typedef struct res2tac_tuning {
 /* Validates *p, allocates the context's device scratch for a W x H x D pair on the current
  * device, and returns the handle in *out. The scratch (cost volume, aggregated
  * volume, intermediate maps, host staging) is owned by the context until res2tac_destroy.
+ * Where p2 <= 255, the cost is the census, the scratch stays below 32 GB (W H D below 2^32) and at
+ * least half of the device's memory stays free with it, the context keeps the paths' terms as byte
+ * planes instead of one volume of sums, which is faster, with identical results: 1 + num_paths / 2
+ * bytes per W*H*D with 2 p2 <= 255, else 1 + num_paths (3 with sums, 5 with 32-bit ones), and 4 B
+ * more per pixel. Otherwise it allocates res2tac_workspace_bytes.
  * Returns RES2TAC_EINVAL for invalid parameters, RES2TAC_ENOMEM if the scratch does not fit. */
 int res2tac_create(const res2tac_params* p, res2tac_t* out);
 
@@ -229,7 +236,9 @@ int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res
 int res2tac_debug_outputs(res2tac_t h, uint8_t* cost, uint16_t* agg, uint16_t* dl, uint16_t* dr,
                           uint8_t* mask, res2tac_stream_t s);
 
-/* Device bytes res2tac_create allocates for *p (0 if *p is invalid); for admission control. */
+/* Device bytes a context for *p needs (0 if *p is invalid); for admission control. It takes more,
+ * for path planes, only where at least half of the device's memory stays free (see
+ * res2tac_create). */
 size_t res2tac_workspace_bytes(const res2tac_params* p);
 
 /* Device bytes a batch of n pairs needs on top of the context (0 if a pair is invalid). */
@@ -315,7 +324,7 @@ int res2tac_stage_times(res2tac_t h, float* ms, int n);
  * 5 B per W*H*D when num_paths * (255 + p2) > 65535, 4 B more per pixel with RES2TAC_EXACT_CC,
  * 24 B more per pixel and 2 KB with RES2TAC_NCC)
  * is rejected with RES2TAC_ENOMEM and a
- * message giving both sizes. 640 x 480 with D = 64 fits with 16-bit sums
+ * message giving both sizes. Where it fits, the array holds path planes (see res2tac_create). 640 x 480 with D = 64 fits with 16-bit sums
  * (num_paths * (255 + p2) <= 65535: about 67 MB) but not with 32-bit ones (about 106 MB).
  * Set-up: the first call on a device looks up the array's device address (cudaGetSymbolAddress)
  * with that device current; make that first call before any stream capture.

@@ -93,6 +93,7 @@ struct res2tac_ctx {
   float* maps;         // rectification maps mapx_l, mapy_l, mapx_r, mapy_r (W x H each), or NULL
   int raw_w, raw_h;    // raw image size the maps sample
   int last_launches;
+  int last_planar;     // the last call left path planes (else one volume of sums)
   r2t::BatchEngine* batch;
   int profiling;
   cudaEvent_t ev[8];  // stage boundaries of the last profiled compute (8 with the exact check)
@@ -118,9 +119,8 @@ const char* res2tac_last_error(void) { return g_err; }
 size_t res2tac_workspace_bytes(const res2tac_params* p) {
   if (params_error(p)) return 0;
   const size_t npx = (size_t)p->width * p->height;
-  return layout_for(p->width, p->height, p->max_disp, needs_wide(p),
-                    (p->flags & RES2TAC_EXACT_CC) != 0, (p->flags & RES2TAC_NCC) != 0).total +
-         npx * 2 + npx * 2 + 1024;
+  return r2t::layout_single(p->width, p->height, p->max_disp, method_of(*p), 0).total + npx * 2 +
+         npx * 2 + 1024;
 }
 
 int res2tac_create(const res2tac_params* p, res2tac_t* out) {
@@ -132,16 +132,24 @@ int res2tac_create(const res2tac_params* p, res2tac_t* out) {
   memset(h, 0, sizeof(*h));
   h->p = *p;
   h->method = method_of(*p);
-  h->tuning = r2t::default_tuning(p->max_disp);
   cudaError_t e = cudaGetDevice(&h->device);
   if (e != cudaSuccess) {
     delete h;
     return fail_cuda(e, "cudaGetDevice");
   }
-  h->lay = layout_for(p->width, p->height, p->max_disp, h->method.wide != 0,
-                      (p->flags & RES2TAC_EXACT_CC) != 0, (p->flags & RES2TAC_NCC) != 0);
+  // path planes only where half of the device's memory stays free with them
   const size_t npx = (size_t)p->width * p->height;
-  e = cudaMalloc(&h->scratch, h->lay.total);
+  size_t free_b = 0, total_b = 0;
+  h->lay = r2t::layout_single(p->width, p->height, p->max_disp, h->method);
+  if (h->lay.planes && (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
+                        h->lay.total + 4 * npx + total_b / 2 > free_b ||
+                        cudaMalloc(&h->scratch, h->lay.total) != cudaSuccess)) {
+    cudaGetLastError();
+    h->lay = r2t::layout_single(p->width, p->height, p->max_disp, h->method, 0);
+    h->scratch = nullptr;
+  }
+  if (!h->scratch) e = cudaMalloc(&h->scratch, h->lay.total);
+  h->tuning = r2t::default_tuning(p->max_disp, h->lay.planes != 0);
   if (e == cudaSuccess) e = cudaMemset(h->scratch + h->lay.fault, 0, 16);  // range-check record
   if (e == cudaSuccess) e = cudaMalloc(&h->stage_in, align_up(npx * 2, 256));
   if (e == cudaSuccess) e = cudaMalloc(&h->stage_out, align_up(npx * 2, 256));
@@ -172,6 +180,23 @@ void res2tac_destroy(res2tac_t h) {
   delete h;
 }
 
+// The context's problem for one call: on path planes where the scratch has them and the settings
+// allow it (the planes' memory also holds the volume of sums otherwise).
+static r2t::Problem call_problem(res2tac_t h, bool subpixel) {
+  r2t::Problem pb = problem_at(h->scratch, h->lay, h->p.width, h->p.height, h->p.max_disp);
+  pb.planar = pb.planar && r2t::planar_tuning(h->tuning);
+  if (!subpixel || !pb.planar) pb.dlf = nullptr;
+  h->last_planar = pb.planar;
+  return pb;
+}
+
+// The problem the last call left, for the debug copies.
+static r2t::Problem last_problem(res2tac_t h) {
+  r2t::Problem pb = problem_at(h->scratch, h->lay, h->p.width, h->p.height, h->p.max_disp);
+  pb.planar = h->last_planar;
+  return pb;
+}
+
 static int check_io(res2tac_t h, const void* left, const void* right, int64_t in_pitch,
                     const void* disp, int64_t out_pitch) {
   if (!h) return fail(RES2TAC_EINVAL, "handle is NULL");
@@ -188,7 +213,7 @@ int res2tac_compute(res2tac_t h, const uint8_t* left, const uint8_t* right, int6
                     uint16_t* disp, int64_t out_pitch, res2tac_stream_t s) {
   int rc = check_io(h, left, right, in_pitch, disp, out_pitch);
   if (rc) return rc;
-  r2t::Problem pb = problem_at(h->scratch, h->lay, h->p.width, h->p.height, h->p.max_disp);
+  r2t::Problem pb = call_problem(h, false);
   pb.left = left;
   pb.right = right;
   pb.in_pitch = in_pitch;
@@ -330,7 +355,7 @@ int res2tac_compute_subpixel(res2tac_t h, const uint8_t* left, const uint8_t* ri
     return fail(RES2TAC_EINVAL, "out_pitch must be a multiple of 4 and >= 4 * width");
   if ((reinterpret_cast<uintptr_t>(disp) & 3) != 0)
     return fail(RES2TAC_EINVAL, "disp must be 4-byte aligned");
-  r2t::Problem pb = problem_at(h->scratch, h->lay, h->p.width, h->p.height, h->p.max_disp);
+  r2t::Problem pb = call_problem(h, true);
   pb.left = left;
   pb.right = right;
   pb.in_pitch = in_pitch;
@@ -347,8 +372,8 @@ int res2tac_compute_subpixel(res2tac_t h, const uint8_t* left, const uint8_t* ri
 
 int res2tac_debug_subpixel(res2tac_t h, float* dl_sub, res2tac_stream_t s) {
   if (!h || !dl_sub) return fail(RES2TAC_EINVAL, "NULL argument");
-  r2t::Problem pb = problem_at(h->scratch, h->lay, h->p.width, h->p.height, h->p.max_disp);
-  cudaError_t e = r2t::copy_subpixel(pb, h->method.wide != 0, dl_sub, (cudaStream_t)s);
+  r2t::Problem pb = last_problem(h);
+  cudaError_t e = r2t::copy_subpixel(pb, h->method, dl_sub, (cudaStream_t)s);
   if (e != cudaSuccess) return fail_cuda(e, "res2tac_debug_subpixel");
   return RES2TAC_OK;
 }
@@ -356,12 +381,12 @@ int res2tac_debug_subpixel(res2tac_t h, float* dl_sub, res2tac_stream_t s) {
 int res2tac_debug_outputs(res2tac_t h, uint8_t* cost, uint16_t* agg, uint16_t* dl, uint16_t* dr,
                           uint8_t* mask, res2tac_stream_t s) {
   if (!h) return fail(RES2TAC_EINVAL, "handle is NULL");
-  r2t::Problem pb = problem_at(h->scratch, h->lay, h->p.width, h->p.height, h->p.max_disp);
+  r2t::Problem pb = last_problem(h);
   cudaStream_t st = (cudaStream_t)s;
   const size_t npx = (size_t)pb.W * pb.H;
   cudaError_t e = cudaSuccess;
   if (cost && e == cudaSuccess) e = r2t::copy_cost(pb, cost, st);
-  if (agg && e == cudaSuccess) e = r2t::copy_agg_u16(pb, h->method.wide != 0, agg, st);
+  if (agg && e == cudaSuccess) e = r2t::copy_agg_u16(pb, h->method, agg, st);
   if (dl && e == cudaSuccess) e = cudaMemcpyAsync(dl, pb.dl, npx * 2, cudaMemcpyDeviceToDevice, st);
   if (dr && e == cudaSuccess) e = cudaMemcpyAsync(dr, pb.dr, npx * 2, cudaMemcpyDeviceToDevice, st);
   if (mask && e == cudaSuccess) e = cudaMemcpyAsync(mask, pb.mask, npx, cudaMemcpyDeviceToDevice, st);
@@ -384,7 +409,7 @@ int res2tac_get_tuning(res2tac_t h, res2tac_tuning* t) {
 
 int res2tac_set_tuning(res2tac_t h, const res2tac_tuning* t) {
   if (!h || !t) return fail(RES2TAC_EINVAL, "NULL argument");
-  r2t::Tuning n = r2t::default_tuning(h->p.max_disp);
+  r2t::Tuning n = r2t::default_tuning(h->p.max_disp, h->lay.planes != 0);
   if (t->agg_dpl) n.agg_dpl = t->agg_dpl;
   if (t->agg_warps) n.agg_warps = t->agg_warps;
   if (t->wta_chunk) n.wta_chunk = t->wta_chunk;

@@ -142,7 +142,7 @@ __device__ __forceinline__ uint32_t group_min(uint32_t v) {
         const uint32_t v1 = __shfl_xor_sync(0xffffffffu, v, a, LPL);
         const uint32_t v2 = __shfl_xor_sync(0xffffffffu, v, 2 * a, LPL);
         const uint32_t v3 = __shfl_xor_sync(0xffffffffu, v, 3 * a, LPL);
-        v = vmin2(vmin2(v, v1), vmin2(v2, v3));
+        v = vmin2(__vimin3_u16x2(v, v1, v2), v3);
       } else {
         v = vmin2(v, __shfl_xor_sync(0xffffffffu, v, a, LPL));
       }

@@ -41,7 +41,7 @@ struct CensusSmem {
 // words are 4 disparities apart), which this split keeps on consecutive words (no bank conflict).
 struct CostSmem {
   uint64_t l[kCostTX];                // CT_L(x0 .. x0 + kCostTX - 1)
-  uint64_t r[4][(kCostTX + 256) / 4]; // CT_R(x0 - D + i), i < kCostTX + D (0 outside the image)
+  uint64_t r[4][(kCostTX + 256) / 4 + 1]; // CT_R(x0 - D + i), i < kCostTX + D (0 outside the image)
 };
 
 // Bytewise unsigned a < b of four byte lanes, in bit 7 of each byte (other bits undefined).
@@ -268,6 +268,77 @@ __device__ __forceinline__ void cost_tile(const Problem& pb, int item, CostSmem&
                                         ((int64_t)y * W + x0) * D * agg_bytes_per_de);
     for (int i = threadIdx.x; i < nv; i += blockDim.x) z[i] = make_uint4(0, 0, 0, 0);
     for (int i = threadIdx.x; i < npx; i += blockDim.x) pb.kr[(int64_t)y * W + x0 + i] = 0xFFFFFFFFu;
+  }
+  __syncthreads();
+}
+
+// One row segment of kCostTX pixels in the pair order of the path planes (planar.cuh): thread t
+// computes the 8 costs d = 4q .. 4q + 3 and D/2 + 4q .. D/2 + 4q + 3 (8 adjacent bytes), q = t %
+// (D/8), over a run of consecutive pixels; of the two windows of four right descriptors three
+// carry over in registers from one pixel to the next. Runs are a multiple of 4 pixels long, so
+// a descriptor's phase is a compile-time offset. The tile's right-disparity keys are reset.
+template <bool CT64>
+__device__ __forceinline__ void cost_tile_planar(const Problem& pb, int item, CostSmem& sm) {
+  const int ntx = (pb.W + kCostTX - 1) / kCostTX;
+  const int y = item / ntx;
+  const int x0 = (item - y * ntx) * kCostTX;
+  const int W = pb.W, D = pb.D, h = D / 2;
+  const int npx = min(kCostTX, W - x0);
+  const uint64_t* ctl = pb.ct + (int64_t)y * W;
+  const uint64_t* ctr = pb.ct + (int64_t)W * pb.H + (int64_t)y * W;
+  for (int i = threadIdx.x; i < kCostTX + D; i += blockDim.x) {
+    if (i < kCostTX) sm.l[i] = i < npx ? ctl[x0 + i] : 0ull;
+    const int xr = x0 - D + i;  // only x - d >= 0 within the row are read
+    sm.r[i & 3][i >> 2] = (xr >= 0 && xr < W) ? ctr[xr] : 0ull;
+  }
+  for (int i = threadIdx.x; i < npx; i += blockDim.x)
+    pb.kr[(int64_t)y * W + x0 + i] = 0xFFFFFFFFu;
+  __syncthreads();
+  const int nq = D / 8, runs = 256 / nq;
+  const int ppr = ((kCostTX + runs - 1) / runs + 3) & ~3;
+  const int run = threadIdx.x / nq, q = threadIdx.x - run * nq, px0 = run * ppr;
+  if (run < runs && px0 < npx) {
+    int aw = (px0 + D - 4 * q) >> 2, bw = aw - h / 4;  // words of phase 0
+#define R2T_RD(w, o) sm.r[(o) & 3][(w) + ((o) >> 2)]
+    uint64_t a0 = R2T_RD(aw, 0), a1 = R2T_RD(aw, -1), a2 = R2T_RD(aw, -2), a3 = R2T_RD(aw, -3);
+    uint64_t b0 = R2T_RD(bw, 0), b1 = R2T_RD(bw, -1), b2 = R2T_RD(bw, -2), b3 = R2T_RD(bw, -3);
+    uint2* o = reinterpret_cast<uint2*>(pb.cost + ((int64_t)y * W + x0 + px0) * D + 8 * q);
+    const bool interior = x0 >= D - 1;  // block-uniform
+    const int end = min(ppr, npx - px0);
+    const uint64_t *l = sm.l + px0;
+    // whole groups of 4 pixels are computed (their reads stay inside sm), the stores are tested
+    for (int kb = 0; kb < end; kb += 4, l += 4, aw++, bw++) {
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const uint64_t cl = l[k];
+        uint32_t u0 = hamming<CT64>(cl, a0), u1 = hamming<CT64>(cl, a1);
+        uint32_t u2 = hamming<CT64>(cl, a2), u3 = hamming<CT64>(cl, a3);
+        uint32_t v0 = hamming<CT64>(cl, b0), v1 = hamming<CT64>(cl, b1);
+        uint32_t v2 = hamming<CT64>(cl, b2), v3 = hamming<CT64>(cl, b3);
+        if (!interior) {  // x - d < 0: outside the right image
+          const int m = x0 + px0 + kb + k - 4 * q;
+          u0 = m < 0 ? kCostOutside : u0;
+          u1 = m < 1 ? kCostOutside : u1;
+          u2 = m < 2 ? kCostOutside : u2;
+          u3 = m < 3 ? kCostOutside : u3;
+          v0 = m < h ? kCostOutside : v0;
+          v1 = m < h + 1 ? kCostOutside : v1;
+          v2 = m < h + 2 ? kCostOutside : v2;
+          v3 = m < h + 3 ? kCostOutside : v3;
+        }
+        if (kb + k < end) o[(kb + k) * nq] = make_uint2(pack_bytes(u0, v0, u1, v1), pack_bytes(u2, v2, u3, v3));
+        // one pixel right: both windows move by one descriptor
+        a3 = a2;
+        a2 = a1;
+        a1 = a0;
+        a0 = R2T_RD(aw, k + 1);
+        b3 = b2;
+        b2 = b1;
+        b1 = b0;
+        b0 = R2T_RD(bw, k + 1);
+      }
+    }
+#undef R2T_RD
   }
   __syncthreads();
 }

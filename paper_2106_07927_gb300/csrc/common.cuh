@@ -39,6 +39,9 @@ struct Problem {
   uint16_t* dp;       // [H][W] D^L of that swapped, flipped pair (exact check); NULL: approximate
   uint2* nst;         // [2][H][W] patch sum and factor of the reference / matching image (NCC)
   int32_t* nsv;       // [2][H][W] exact patch variance N sum a^2 - (sum a)^2 of both images (NCC)
+  int planar;         // agg holds the paths' byte planes (see planar.cuh), cost is in pair order
+  int64_t plane;      // bytes of one plane (W H D)
+  float* dlf;         // [H][W] sub-pixel D^L of a planar sub-pixel call; NULL: not computed
   unsigned* fault;    // range-check record {site, 0, byte offset (int64)} (RES2TAC_CHECK_BOUNDS)
 };
 
@@ -49,6 +52,7 @@ struct Problem {
 // constant true and compiles away.
 // Sites: 1 row-kernel cost load, 2 row-kernel add into S, 3 sheared-kernel cost copy, 4 / 5
 // sheared-kernel bulk add (run before / after a wrap), 6 WTA staging copy of S, 7 WTA store of D^L.
+// (planes: 3 also the own-lane cost copies, 2 and 4 the stores of U)
 // Site 8 is recorded in every build: a block of the tensor-core cost kernel whose MMAs did not
 // complete within its poll limit (it stores no cost).
 #ifdef RES2TAC_CHECK_BOUNDS

@@ -6,6 +6,7 @@
 #include "aggregate.cuh"
 #include "census_cost.cuh"
 #include "launch.h"
+#include "planar.cuh"
 #include "post.cuh"
 
 namespace r2t {
@@ -18,6 +19,20 @@ __global__ void __launch_bounds__(256) census_kernel(Problem pb, Method mt) {
 __global__ void __launch_bounds__(256) cost_kernel(Problem pb, Method mt) {
   __shared__ CostSmem sm;
   cost_tile_dispatch(pb, mt, blockIdx.x, sm);
+}
+
+__global__ void __launch_bounds__(256) cost_planar_kernel(Problem pb, Method mt) {
+  __shared__ CostSmem sm;
+  if (mt.cw == 9)
+    cost_tile_planar<true>(pb, blockIdx.x, sm);
+  else
+    cost_tile_planar<false>(pb, blockIdx.x, sm);
+}
+
+template <int R>
+__global__ void __launch_bounds__(256) wta_planar_kernel(Problem pb, int paths, int T) {
+  extern __shared__ __align__(16) uint8_t wsm[];
+  planar_wta_tile<R>(pb, paths, blockIdx.x, wsm, T);
 }
 
 template <bool WIDE>
@@ -41,8 +56,45 @@ __global__ void subpixel_map_kernel(Problem pb, float* out) {
     out[i] = refine_subpixel<WIDE>(pb, i, pb.dl[i]);
 }
 
-cudaError_t copy_subpixel(const Problem& pb, bool wide, float* dst, cudaStream_t s) {
-  if (wide)
+// S(p, d) of pair order volumes: the cost times the path count plus the planes.
+__device__ __forceinline__ uint32_t planar_sum(const Problem& pb, const Method& mt, int64_t p,
+                                               int d) {
+  const int h = pb.D / 2;
+  const int64_t i = p * pb.D + (d < h ? 2 * d : 2 * (d - h) + 1);
+  uint32_t s = mt.num_paths * pb.cost[i];
+  for (int r = 0; r < planar_planes(mt); r++)
+    s += reinterpret_cast<const uint8_t*>(pb.agg)[r * pb.plane + i];
+  return s;
+}
+
+// Debug copies of the planar volumes in natural order: the sums, the cost and the sub-pixel D^L.
+__global__ void planar_copy_kernel(Problem pb, Method mt, uint16_t* agg, uint8_t* cost,
+                                   float* sub) {
+  const int64_t n = sub ? (int64_t)pb.W * pb.H : pb.plane;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (sub) {
+      const int d = pb.dl[i];
+      float v = (float)d;
+      if (d >= 1 && d <= pb.D - 2) {
+        const int s0 = (int)planar_sum(pb, mt, i, d), a = (int)planar_sum(pb, mt, i, d - 1) - s0;
+        const int b = (int)planar_sum(pb, mt, i, d + 1) - s0;
+        v = __fadd_rn(v, __fdiv_rn((float)(a - b), (float)(2 * (a + b))));
+      }
+      sub[i] = v;
+      continue;
+    }
+    const int64_t p = i / pb.D;
+    const int d = (int)(i - p * pb.D), h = pb.D / 2;
+    if (agg) agg[i] = (uint16_t)planar_sum(pb, mt, p, d);
+    if (cost) cost[i] = pb.cost[p * pb.D + (d < h ? 2 * d : 2 * (d - h) + 1)];
+  }
+}
+
+cudaError_t copy_subpixel(const Problem& pb, const Method& mt, float* dst, cudaStream_t s) {
+  if (pb.planar)
+    planar_copy_kernel<<<608, 256, 0, s>>>(pb, mt, nullptr, nullptr, dst);
+  else if (mt.wide)
     subpixel_map_kernel<true><<<608, 256, 0, s>>>(pb, dst);
   else
     subpixel_map_kernel<false><<<608, 256, 0, s>>>(pb, dst);
@@ -60,7 +112,7 @@ __global__ void agg_copy_kernel(const void* src, uint16_t* dst, int64_t n) {
   }
 }
 
-Tuning default_tuning(int D) {
+Tuning default_tuning(int D, bool planar) {
   Tuning t;
   t.agg_dpl = long_dpl_default(D);
   t.agg_warps = 2;  // two warps per block (measured best with one row direction per lane group)
@@ -70,6 +122,12 @@ Tuning default_tuning(int D) {
   t.row_split = 1;  // one row direction per lane group (measured 2 % faster at D = 128)
   t.cost_mode = 0;  // population counts: measured faster than the tensor-core kernel
   t.row_cost = 0;   // the row kernel reads the cost volume
+  if (planar) {
+    // 1242 x 375, D = 128: 0.158 ms for the stage with one chain per lane, 0.173 with two;
+    // selection tiles of 64 pixels 0.051 ms, of 128 0.057 (1920 x 1080, D = 256: 0.455, 0.480)
+    t.shear_cpl = 1;
+    t.wta_chunk = 64;
+  }
   return t;
 }
 
@@ -114,6 +172,12 @@ void fork_destroy(Fork* f) {
 
 static cudaError_t launch_aggregate(const Problem& pb, const Method& mt, const Tuning& tn,
                                     cudaStream_t s, const Fork* fork) {
+  if (pb.planar) {
+    // one stream: the row kernel's blocks, which hold the longest chains, are placed first and
+    // evenly; the sheared kernel's follow beside them (programmatic dependent launch)
+    const cudaError_t e = launch_planar_rows(pb, mt, tn, s);
+    return e != cudaSuccess ? e : launch_planar_shear(pb, mt, tn, s);
+  }
   cudaStream_t ls = s;
   if (fork) {
     cudaEventRecord(fork->fork, s);
@@ -131,6 +195,25 @@ static cudaError_t launch_aggregate(const Problem& pb, const Method& mt, const T
   return cudaGetLastError();
 }
 
+template <int R>
+static cudaError_t launch_planar_wta_t(const Problem& pb, int paths, int T, cudaStream_t s) {
+  const size_t smem = planar_wta_smem(pb.D, T);
+  cudaFuncSetAttribute(wta_planar_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)smem);
+  wta_planar_kernel<R><<<wta_items(pb.W, pb.H, T), 256, smem, s>>>(pb, paths, T);
+  return cudaGetLastError();
+}
+
+static cudaError_t launch_planar_wta(const Problem& pb, const Method& mt, const Tuning& tn,
+                                     cudaStream_t s) {
+  const int T = planar_wta_px(pb.D, tn.wta_chunk);
+  switch (planar_planes(mt)) {
+    case 8: return launch_planar_wta_t<8>(pb, mt.num_paths, T, s);
+    case 4: return launch_planar_wta_t<4>(pb, mt.num_paths, T, s);
+    default: return launch_planar_wta_t<2>(pb, mt.num_paths, T, s);
+  }
+}
+
 // Census + cost (or the NCC cost), aggregation and WTA (with the right-disparity keys) of the
 // pair pb.left / pb.right into pb.dl; adds its launches to *n. ev: NULL, or 3 events recorded
 // after each of the 3 stages.
@@ -145,7 +228,9 @@ static cudaError_t run_pass(const Problem& pb, const Method& mt, const Tuning& t
     *n += 3;
   } else {
     census_kernel<<<2 * census_items(pb.W, pb.H), 256, 0, s>>>(pb, mt);
-    if (tn.cost_mode == 1 && cost_mma_ok(pb, mt)) {
+    if (pb.planar) {
+      cost_planar_kernel<<<cost_items(pb.W, pb.H), 256, 0, s>>>(pb, mt);
+    } else if (tn.cost_mode == 1 && cost_mma_ok(pb, mt)) {
       if ((e = launch_cost_mma(pb, mt, s)) != cudaSuccess) return e;
     } else {
       cost_kernel<<<cost_items(pb.W, pb.H), 256, 0, s>>>(pb, mt);
@@ -161,6 +246,13 @@ static cudaError_t run_pass(const Problem& pb, const Method& mt, const Tuning& t
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[1], s);
   nvtxRangePushA("res2tac wta + right-disparity keys");
+  if (pb.planar) {
+    if ((e = launch_planar_wta(pb, mt, tn, s)) != cudaSuccess) return e;
+    nvtxRangePop();
+    if (ev) cudaEventRecord(ev[2], s);
+    *n += 3;
+    return cudaSuccess;
+  }
   // pixels per block of 256 threads, capped so that the staged sums take at most 64 KB
   const int T = wta_staged_px(pb.D, mt.wide != 0, tn.wta_chunk);
   const size_t smem = wta_staged_smem_bytes(pb.D, mt.wide != 0, T);
@@ -216,6 +308,7 @@ cudaError_t run_pipeline(const Problem& pb, const Method& mt, const Tuning& tn, 
     pf.right = pb.flip + npx;
     pf.in_pitch = pb.W;
     pf.dl = pb.dp;
+    pf.dlf = nullptr;
     if ((e = run_pass(pf, mt, tn, s, ev ? ev + 1 : nullptr, fork, &n)) != cudaSuccess) return e;
   }
   if ((e = run_pass(pb, mt, tn, s, ev ? ev + (exact ? 4 : 1) : nullptr, fork, &n)) !=
@@ -237,9 +330,11 @@ cudaError_t run_pipeline(const Problem& pb, const Method& mt, const Tuning& tn, 
   return cudaSuccess;
 }
 
-cudaError_t copy_agg_u16(const Problem& pb, bool wide, uint16_t* dst, cudaStream_t s) {
+cudaError_t copy_agg_u16(const Problem& pb, const Method& mt, uint16_t* dst, cudaStream_t s) {
   const int64_t n = (int64_t)pb.W * pb.H * pb.D;
-  if (wide)
+  if (pb.planar)
+    planar_copy_kernel<<<1216, 256, 0, s>>>(pb, mt, dst, nullptr, nullptr);
+  else if (mt.wide)
     agg_copy_kernel<true><<<1216, 256, 0, s>>>(pb.agg, dst, n);
   else
     agg_copy_kernel<false><<<1216, 256, 0, s>>>(pb.agg, dst, n);
@@ -247,6 +342,10 @@ cudaError_t copy_agg_u16(const Problem& pb, bool wide, uint16_t* dst, cudaStream
 }
 
 cudaError_t copy_cost(const Problem& pb, uint8_t* dst, cudaStream_t s) {
+  if (pb.planar) {
+    planar_copy_kernel<<<1216, 256, 0, s>>>(pb, Method(), nullptr, dst, nullptr);
+    return cudaGetLastError();
+  }
   return cudaMemcpyAsync(dst, pb.cost, (size_t)pb.W * pb.H * pb.D, cudaMemcpyDeviceToDevice, s);
 }
 

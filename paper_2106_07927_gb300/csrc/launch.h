@@ -27,8 +27,8 @@ struct Fork {
 cudaError_t fork_create(Fork* f);
 void fork_destroy(Fork* f);
 
-// Default configuration for a disparity count D.
-Tuning default_tuning(int D);
+// Default configuration for a disparity count D; planar: of the path-plane kernels.
+Tuning default_tuning(int D, bool planar = false);
 // True when the configuration can run a pair with D disparities.
 bool tuning_valid(const Tuning& t, int D);
 
@@ -38,6 +38,38 @@ template <bool WIDE>
 cudaError_t launch_rows(const Problem& pb, const Method& mt, const Tuning& tn, cudaStream_t s);
 template <bool WIDE>
 cudaError_t launch_shear(const Problem& pb, const Method& mt, const Tuning& tn, cudaStream_t s);
+// The two kernels on path planes (pb.planar; defined in the agg_planar_*.cu units).
+cudaError_t launch_planar_rows(const Problem& pb, const Method& mt, const Tuning& tn,
+                               cudaStream_t s);
+cudaError_t launch_planar_shear(const Problem& pb, const Method& mt, const Tuning& tn,
+                                cudaStream_t s);
+// Launches a kernel of the aggregation with the SM's memory split for the most shared memory: a
+// block is placed beside blocks of another kernel only when both ask for the same split. With the
+// driver's own choice the sheared kernel's blocks waited for the row kernel's to leave (1242 x
+// 375, D = 128: started at 75 us, on 118 of the SMs). dependent: may start its blocks as soon as
+// every block of the kernel before it has called launch_dependents.
+template <class... P, class... A>
+inline cudaError_t launch_agg(void (*kernel)(P...), int grid, int threads, size_t smem,
+                              cudaStream_t s, bool dependent, A... args) {
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[0].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = dependent ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+// Settings the plane kernels have (blocks are always one pair of warps): 16 disparities per lane of the sheared chains, one row
+// direction per lane group, costs from the volume of the population-count kernel.
+inline bool planar_tuning(const Tuning& tn) {
+  return tn.shear_dpl == 16 && tn.row_split == 1 && tn.cost_mode == 0 && tn.row_cost == 0;
+}
 // Persistent batch variants of the two kernels, as handles for cudaLaunchKernel. Parameters:
 // (const BatchHeader*, const GroupDesc*, const Problem*, const AggSeg* segs,
 // const int* seg_prefix, Method, unsigned* counters, int warp_smem); 256 threads; the sheared
@@ -105,9 +137,9 @@ cudaError_t probe_popc_rate(int iters, cudaStream_t s, double* popc_per_s);
 cudaError_t probe_red_peak(int64_t bytes, int passes, cudaStream_t s, double* bytes_per_s);
 
 // Copies the aggregated volume as saturated uint16 / the cost volume, both in natural order.
-cudaError_t copy_agg_u16(const Problem& pb, bool wide, uint16_t* dst, cudaStream_t s);
+cudaError_t copy_agg_u16(const Problem& pb, const Method& mt, uint16_t* dst, cudaStream_t s);
 cudaError_t copy_cost(const Problem& pb, uint8_t* dst, cudaStream_t s);
-// Writes the sub-pixel D^L map of the last sub-pixel run (float [H][W]).
-cudaError_t copy_subpixel(const Problem& pb, bool wide, float* dst, cudaStream_t s);
+// Writes the sub-pixel D^L map of the last run (float [H][W]).
+cudaError_t copy_subpixel(const Problem& pb, const Method& mt, float* dst, cudaStream_t s);
 
 }  // namespace r2t

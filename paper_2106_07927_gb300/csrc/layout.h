@@ -8,23 +8,33 @@
 namespace r2t {
 
 struct Layout {
-  size_t cost, ct, agg, dl, dr, kr, mask, flip, dp, nst, nsv, fault, total;  // 0: buffer not used
+  size_t cost, ct, agg, dl, dr, kr, mask, flip, dp, nst, nsv, dlf, fault, total;  // 0: not used
+  int planes;  // byte planes agg holds (the path count) instead of one volume of sums, or 0
 };
 
 inline size_t align256(size_t v) { return (v + 255) / 256 * 256; }
+
+// Largest scratch a pair may take with path planes (5 or 9 B per DE instead of 3): an eighth of the
+// device's memory, and volumes below 4 GB (the plane kernels keep 32-bit offsets). 3840 x 2160 with
+// D = 256 takes 10.9 or 19.3 GB; larger pairs keep the small layout, so whatever fitted the
+// device still does.
+constexpr size_t kPlanarBytes = (size_t)32 << 30;
 
 // Cost 1 B/DE, aggregated volume 2 B/DE (4 when wide), census descriptors of both images
 // 16 B/px, D^L and D^R 2 B/px each, right-disparity keys 4 B/px, LR mask 1 B/px: 3 B per DE +
 // 25 B per pixel. The exact
 // consistency check adds the swapped, flipped pair (2 B/px) and its D^L (2 B/px); the NCC cost
-// the patch statistics of both images (16 B/px) and their exact patch variances (8 B/px).
-inline Layout layout_for(int W, int H, int D, bool wide, bool exact = false, bool ncc = false) {
+// the patch statistics of both images (16 B/px) and their exact patch variances (8 B/px). With
+// planes > 0 the aggregated volume is that many byte planes, and the sub-pixel D^L takes 4 B/px.
+inline Layout layout_for(int W, int H, int D, bool wide, bool exact = false, bool ncc = false,
+                         int planes = 0) {
   const size_t npx = (size_t)W * H, nde = npx * D;
   Layout l;
   size_t o = 0;
   l.cost = o; o = align256(o + nde);
   l.ct = o; o = align256(o + npx * 16);
-  l.agg = o; o = align256(o + nde * (wide ? 4 : 2));
+  l.planes = planes;
+  l.agg = o; o = align256(o + nde * (planes ? planes : (wide ? 4 : 2)));
   l.dl = o; o = align256(o + npx * 2);
   l.dr = o; o = align256(o + npx * 2);
   l.kr = o; o = align256(o + npx * 4);
@@ -35,6 +45,8 @@ inline Layout layout_for(int W, int H, int D, bool wide, bool exact = false, boo
     l.flip = o; o = align256(o + npx * 2);
     l.dp = o; o = align256(o + npx * 2);
   }
+  l.dlf = 0;
+  if (planes) { l.dlf = o; o = align256(o + npx * 4); }
   l.nst = l.nsv = 0;
   if (ncc) {  // 2 KB of slack in front (reads at a matching pixel x - d < 0 stay inside)
     l.nst = o + 2048; o = align256(o + 2048 + npx * 16);
@@ -42,6 +54,18 @@ inline Layout layout_for(int W, int H, int D, bool wide, bool exact = false, boo
   }
   l.total = o;
   return l;
+}
+
+// The layout of a pair processed alone: path planes where the method's U fits a byte (census cost,
+// P2 <= 255) and the scratch stays within limit, else one volume of sums.
+inline Layout layout_single(int W, int H, int D, const Method& m, size_t limit = kPlanarBytes) {
+  const bool exact = (m.flags & 4) != 0, ncc = (m.flags & 8) != 0;
+  if (m.P2 <= 255 && !ncc && (size_t)W * H * D < ((size_t)1 << 32) - 65536) {
+    const Layout l =
+        layout_for(W, H, D, false, exact, false, 2 * m.P2 <= 255 ? m.num_paths / 2 : m.num_paths);
+    if (l.total <= limit) return l;
+  }
+  return layout_for(W, H, D, m.wide != 0, exact, ncc);
 }
 
 inline Problem problem_at(char* base, const Layout& l, int W, int H, int D) {
@@ -62,6 +86,9 @@ inline Problem problem_at(char* base, const Layout& l, int W, int H, int D) {
   pb.dp = l.dp ? reinterpret_cast<uint16_t*>(base + l.dp) : nullptr;
   pb.nst = l.nst ? reinterpret_cast<uint2*>(base + l.nst) : nullptr;
   pb.nsv = l.nsv ? reinterpret_cast<int32_t*>(base + l.nsv) : nullptr;
+  pb.planar = l.planes ? 1 : 0;
+  pb.plane = (int64_t)W * H * D;
+  pb.dlf = l.dlf ? reinterpret_cast<float*>(base + l.dlf) : nullptr;
   pb.fault = reinterpret_cast<unsigned*>(base + l.fault);
   return pb;
 }

@@ -45,9 +45,18 @@ extern "C" int res2tac_compute_static(const res2tac_params* p, const uint8_t* le
     return reject(RES2TAC_EINVAL, "res2tac_compute_static: bad pitch or output alignment");
   const int W = p->width, H = p->height, D = p->max_disp;
   const bool wide = p->num_paths * (255 + p->p2) > 65535;
+  r2t::Method mt;
+  mt.cw = p->census_w;
+  mt.ch = p->census_h;
+  mt.P1 = p->p1;
+  mt.P2 = p->p2;
+  mt.num_paths = p->num_paths;
+  mt.flags = p->flags;
+  mt.lr_threshold = p->lr_threshold;
+  mt.wide = wide ? 1 : 0;
   // the same buffers a context allocates, at their offsets inside the array
-  const r2t::Layout lay = r2t::layout_for(W, H, D, wide, (p->flags & RES2TAC_EXACT_CC) != 0,
-                                          (p->flags & RES2TAC_NCC) != 0);
+  // (path planes where they fit it)
+  const r2t::Layout lay = r2t::layout_single(W, H, D, mt, RES2TAC_STATIC_SCRATCH_BYTES);
   if (lay.total > RES2TAC_STATIC_SCRATCH_BYTES)
     return reject(RES2TAC_ENOMEM,
                   "res2tac_compute_static: %dx%d with D=%d needs %zu bytes of scratch, more than "
@@ -80,17 +89,9 @@ extern "C" int res2tac_compute_static(const res2tac_params* p, const uint8_t* le
   pb.in_pitch = in_pitch;
   pb.disp = disp;
   pb.out_pitch = out_pitch;
-  r2t::Method mt;
-  mt.cw = p->census_w;
-  mt.ch = p->census_h;
-  mt.P1 = p->p1;
-  mt.P2 = p->p2;
-  mt.num_paths = p->num_paths;
-  mt.flags = p->flags;
-  mt.lr_threshold = p->lr_threshold;
-  mt.wide = wide ? 1 : 0;
+  pb.dlf = nullptr;
   int launches = 0;
-  e = r2t::run_pipeline(pb, mt, r2t::default_tuning(D), (cudaStream_t)s, &launches, nullptr);
+  e = r2t::run_pipeline(pb, mt, r2t::default_tuning(D, pb.planar != 0), (cudaStream_t)s, &launches, nullptr);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return reject(RES2TAC_ECUDA, "res2tac_compute_static: launch failed: %s",

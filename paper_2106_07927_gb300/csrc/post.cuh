@@ -228,7 +228,8 @@ __device__ __forceinline__ uint32_t checked_from(const Problem& pb, const Method
     const int diff = dl - dr;
     if ((diff < 0 ? -diff : diff) > mt.lr_threshold) return inv;
   }
-  return SUB ? __float_as_uint(refine_subpixel<WIDE>(pb, row + x, dl)) : (uint32_t)dl;
+  if (!SUB) return (uint32_t)dl;
+  return __float_as_uint(pb.dlf ? pb.dlf[row + x] : refine_subpixel<WIDE>(pb, row + x, dl));
 }
 template <bool SUB, bool WIDE>
 __device__ __forceinline__ uint32_t checked_disp(const Problem& pb, const Method& mt, int x, int y) {

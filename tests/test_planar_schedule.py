@@ -1,0 +1,136 @@
+"""Host models of the walks on path planes (csrc/planar.cuh): every cost copy and every store of a
+sheared chain, with its restarts, against the chain definition; the row walk's chunks; and the
+scan ranges of the selection's diagonals against the definition of D^R."""
+import itertools
+
+import pytest
+
+NEVER = 1 << 30
+PF = 6  # steps between a cost copy and its use
+
+
+def _walk(W, H, kind, j, paired):
+    """(copies, stores, restarts) of one chain alone in its warp, pixel by pixel, as the kernel's
+    two pointers and its fast and general pairs of steps make them, in one part or (directions
+    that share a plane) in two; copies are listed by the step that uses them."""
+    sh = 0 if kind < 2 else (1 if kind < 4 else -1)
+    back = kind & 1
+    dy, dx = (-1, -sh) if back else (1, sh)
+    ystart = H - 1 if back else 0
+    x = (j + sh * ystart) % W
+    stride, wrap = dy * W + dx, dx * W
+    wp = ystart * W + x
+    tw = NEVER if dx == 0 else (W - x if dx > 0 else x + 1)
+    copies, stores, restarts = [], [], []
+    base = 0
+    for ph in range(2 if paired else 1):
+        n = H if not paired else (H // 2 if (ph == 0) != bool(back) else H - H // 2)
+        rp, tr = wp, tw
+        tail = 0 if n <= PF + 1 else (n - PF) & ~1
+
+        def copy_step(t):
+            nonlocal rp, tr
+            if t < n:
+                if tr == t:
+                    rp -= wrap
+                    tr += W
+                copies.append(rp)
+                rp += stride
+
+        def next_event(t):
+            return max(min(max(min(tw, tr - PF), 0) & ~1, tail), t)
+
+        for s in range(PF):
+            copy_step(s)
+        te = next_event(0)
+        t = 0
+        while t < n:
+            if t < te:
+                assert t + PF + 1 < n
+                copies += [rp, rp + stride]
+                rp += 2 * stride
+                stores += [wp, wp + stride]
+                wp += 2 * stride
+            else:
+                copy_step(t + PF)
+                copy_step(t + PF + 1)
+                for u in range(2):
+                    if t + u < n:
+                        if tw == t + u:
+                            restarts.append(base + t + u)
+                            wp -= wrap
+                            tw += W
+                        stores.append(wp)
+                        wp += stride
+                te = next_event(t + 2)
+            t += 2
+        tw -= 0 if tw == NEVER else n
+        base += n
+    return copies, stores, restarts
+
+
+@pytest.mark.parametrize("kind", range(6))
+def test_sheared_walk_on_planes(kind):
+    for W, H in itertools.product((1, 2, 3, 5, 8, 13, 40), (1, 2, 5, 6, 7, 8, 9, 14, 15, 33, 100)):
+        sh = 0 if kind < 2 else (1 if kind < 4 else -1)
+        for j in range(W):
+            rows = range(H - 1, -1, -1) if kind & 1 else range(H)
+            want = [y * W + (j + sh * y) % W for y in rows]
+            entry = (0 if sh > 0 else W - 1) if not kind & 1 else (W - 1 if sh > 0 else 0)
+            starts = [t for t, p in enumerate(want) if sh and t and p % W == entry]
+            for paired in (False, True):
+                got = _walk(W, H, kind, j, paired)
+                assert got == (want, want, starts), (W, H, j, paired)
+
+
+@pytest.mark.parametrize("back", [False, True])
+def test_row_walk_chunks(back):
+    G = 8
+    for W, paired in itertools.product(range(1, 60), (False, True)):
+        mid = (W // 2) & ~(G - 1)
+        got, met = [], [0, 0]
+        for ph in range(2 if paired else 1):
+            low = paired and (ph == 0) != back
+            q0, q1 = (mid if paired and not low else 0), (mid if low else W)
+            for k in range((q1 - q0 + G - 1) // G):
+                n = min(G, q1 - q0 - k * G)
+                p = q1 - k * G - n if back else q0 + k * G
+                assert q0 <= p and p + n <= q1
+                got += [p + (n - 1 - u if back else u) for u in range(n)]
+            met[ph] = (q0, q1)
+        assert got == (list(range(W - 1, -1, -1)) if back else list(range(W)))
+        if paired:  # each part covers what the other direction covers in its other part
+            assert met == ([(mid, W), (0, mid)] if back else [(0, mid), (mid, W)])
+
+
+@pytest.mark.parametrize("W,D,T", [(1, 16, 32), (5, 32, 32), (37, 16, 32), (61, 48, 32),
+                                   (80, 64, 64), (70, 256, 32)])
+def test_selection_scans_every_sum_once(W, D, T):
+    # each (pixel, d) with a target x - d >= 0 reaches that target exactly once, and nothing else
+    # does; all word reads stay inside the tile
+    h, pitch = D // 2, D // 2 + 1
+    seen = {}
+    for x0 in range(0, W, T):
+        n = min(T, W - x0)
+        for j in range(n + D - 1):
+            t = j - (D - 1)
+            if x0 + t < 0:
+                continue
+            par = t & 1
+            assert (par - t) % 2 == 0
+            kb, w = (par - t) // 2, par * pitch + (par - t) // 2
+            for _ in range(par, T, 32):
+                for i in range(16):
+                    if 0 <= kb + i < h:
+                        word = w + i * (2 * pitch + 1)
+                        px, k = divmod(word, pitch)
+                        assert 0 <= px < T and k == kb + i
+                        if px < n:  # the other rows hold no sum
+                            # low half d = 2k to target t, high half d = 2k + 1 to target t - 1
+                            # (read by the target's thread from the next diagonal)
+                            seen.setdefault((x0 + px, 2 * k), []).append(x0 + t)
+                            if j >= 1 and x0 + t - 1 >= 0:
+                                seen.setdefault((x0 + px, 2 * k + 1), []).append(x0 + t - 1)
+                kb, w = kb + 16, w + 16 * (2 * pitch + 1)
+    want = {(x, d): [x - d] for x in range(W) for d in range(min(D, x + 1))}
+    assert seen == want
