@@ -213,18 +213,22 @@ int res2tac_compute_raw(res2tac_t h, const uint8_t* raw_left, const uint8_t* raw
                         res2tac_stream_t s);
 
 /* Runs n independent pairs of uneven sizes as one batch on stream s (the paper processes one
- * pair at a time, Sec. 2.2; batching is this library's addition). The pairs are sorted by memory
- * footprint and cut into groups of at most 96 MB of cost and aggregated volumes (a larger pair is
- * a group of its own); each group runs the six stages as persistent kernels fed by device work
- * queues over its pairs, and groups rotate over four stream slots so consecutive groups
- * overlap. The whole batch is one CUDA graph, captured once per group count and replayed while
- * the capacities last (res2tac_last_launch_count: 6 per group). The context grows its batch
- * scratch when a larger batch arrives: that call allocates and must not be made during stream
- * capture. pairs: host array of n descriptors with device pointers. Results are bit-identical to
- * res2tac_compute on each pair alone. No block of the engine ever waits for another (work is
- * claimed with one atomic increment), so there is no device-side wait that could time out:
- * RES2TAC_ETIMEOUT is reserved and not returned. RES2TAC_EINVAL for an invalid pair, or for
- * RES2TAC_EXACT_CC / RES2TAC_NCC contexts (single pairs only). */
+ * pair at a time, Sec. 2.2; batching is this library's addition). Results are bit-identical to
+ * res2tac_compute on each pair alone. pairs: host array of n descriptors with device pointers.
+ * With p2 <= 255 the pairs are cut into groups of one max_disp of at most 96 MB of scratch (a larger
+ * pair is a group of its own); a group runs its six stages with one launch each on path planes
+ * (see res2tac_create), and groups rotate over up to four streams, each with its own part of the
+ * batch scratch, as many as the scratch holds. A pair whose planes do not fit the scratch runs with
+ * its sums in place. Otherwise the groups hold at most 96 MB of cost and aggregated volumes, run
+ * as persistent kernels fed by device work queues and the whole batch is one CUDA graph, captured
+ * once per group count and replayed while the capacities last.
+ * res2tac_last_launch_count: 6 per group. The context grows its batch scratch when a larger batch
+ * arrives (unless res2tac_batch_reserve sized it, to more than res2tac_batch_workspace_bytes only
+ * for a pair's planes and where half of the device's memory stays free): that call allocates and
+ * must not be made during stream capture. No block of either route ever waits for another one of
+ * another launch, so there is no device-side wait that could time out: RES2TAC_ETIMEOUT is reserved
+ * and not returned. RES2TAC_EINVAL for an invalid pair, or for RES2TAC_EXACT_CC / RES2TAC_NCC
+ * contexts (single pairs only). */
 int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res2tac_stream_t s);
 
 /* Copies the intermediates of the last res2tac_compute on this context into caller buffers
@@ -270,7 +274,8 @@ int res2tac_autotune(res2tac_t h, const uint8_t* left, const uint8_t* right, int
  *   shear_dpl, shear_cpl  disparities and chains per lane of the column and diagonal paths:
  *              (16, 1) or (16, 2)
  *   wta_px     pixels per WTA / right-disparity tile: 64, 128 or 256 (fewer when the tile's sums
- *              would exceed 64 KB)
+ *              would exceed 64 KB; half as many on path planes, where shear_dpl and shear_cpl have
+ *              no effect)
  * Defaults: row_dpl 2 / 4 / 8 for D <= 64 / <= 128 / larger, (16, 1), 128. */
 typedef struct res2tac_batch_tuning {
   int32_t max_disp, large;

@@ -95,6 +95,7 @@ struct res2tac_ctx {
   int last_launches;
   int last_planar;     // the last call left path planes (else one volume of sums)
   r2t::BatchEngine* batch;
+  int batch_reserved;  // the batch scratch was sized by res2tac_batch_reserve
   int profiling;
   cudaEvent_t ev[8];  // stage boundaries of the last profiled compute (8 with the exact check)
   r2t::Fork fork;     // second stream for the concurrent aggregation kernels
@@ -573,6 +574,7 @@ size_t res2tac_batch_workspace_bytes(const res2tac_params* p, const res2tac_pair
 int res2tac_batch_reserve(res2tac_t h, size_t scratch_bytes, int32_t max_pairs) {
   if (!h || max_pairs < 1) return fail(RES2TAC_EINVAL, "bad batch reservation");
   int rc = r2t::batch_reserve(&h->batch, scratch_bytes, max_pairs);
+  if (rc == 0) h->batch_reserved = 1;
   if (rc == -2) return fail(RES2TAC_ENOMEM, "batch reservation of %zu bytes failed", scratch_bytes);
   if (rc) return fail(RES2TAC_ECUDA, "batch reservation: %s", r2t::batch_error(h->batch));
   return RES2TAC_OK;
@@ -615,7 +617,11 @@ int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res
     probs[i] = pb;
   }
   int launches = 0;
-  rc = r2t::batch_run(h->batch, probs.data(), n, h->method, (cudaStream_t)s, &launches);
+  if (r2t::batch_planar_method(h->method))
+    rc = r2t::batch_run_planar(h->batch, probs.data(), n, h->method, (cudaStream_t)s,
+                               !h->batch_reserved, &launches);
+  else
+    rc = r2t::batch_run(h->batch, probs.data(), n, h->method, (cudaStream_t)s, &launches);
   h->last_launches = launches;
   if (rc == -4) return fail(RES2TAC_ETIMEOUT, "batch work queue wait timed out");
   if (rc) return fail(RES2TAC_ECUDA, "batch run failed: %s", r2t::batch_error(h->batch));

@@ -25,6 +25,14 @@ char* batch_scratch(BatchEngine* e);
 int batch_run(BatchEngine* e, const Problem* probs, int n, const Method& mt, cudaStream_t s,
               int* launches);
 
+// The route of batches whose method has path planes (batch_planar_method): groups of pairs of one D
+// run stage by stage on up to 4 streams, each stream's groups in one part of the scratch after
+// another. Uses the engine's scratch as it is (grown first to what a lone pair takes when
+// `grow`); a pair whose planes do not fit it runs with its sums in place. Returns 0 or -3.
+bool batch_planar_method(const Method& mt);
+int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& mt, cudaStream_t s,
+                     bool grow, int* launches);
+
 // Kernel settings per bucket of pairs (tune_bucket: D / 16 and the size class): the defaults,
 // their validity, and the engine's table (set returns -1 for an invalid setting).
 BatchTune batch_default_tune(int bucket);

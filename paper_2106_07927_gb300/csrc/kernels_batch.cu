@@ -32,6 +32,8 @@
 #include "batch_dev.cuh"
 #include "census_cost.cuh"
 #include "launch.h"
+#include "layout.h"
+#include "planar_group.h"
 #include "post.cuh"
 
 namespace r2t {
@@ -517,6 +519,140 @@ int batch_run(BatchEngine* e, const Problem* probs, int n, const Method& mt, cud
   if (c != cudaSuccess) return set_err(e, c, "graph launch");
   e->copy_pending = true;
   if (launches) *launches = 6 * G;
+  return 0;
+}
+
+// ------------------------------------------------------------------------------- path planes
+// Batches on path planes: groups of pairs of one D, one launch per stage and group (6), no
+// descriptors in memory and no work queues. Against the persistent kernels above, which add into
+// 16-bit sums: 64 x 320x240, D = 64 1.78 -> 1.34 ms; 16 x 1242x375, D = 128 4.82 -> 3.83 ms; 16
+// uneven pairs up to 1920x1080, D = 256 11.9 -> 7.3 ms.
+// Scratch of one group (a larger pair is a group of its own): 64 x 320x240 took 1.80, 1.34, 1.36 and
+// 1.41 ms with 48, 96, 192 and 400 MB - larger groups fill the GPU, smaller ones stay in the L2;
+// batches of larger pairs do not depend on it.
+constexpr size_t kPlanarGroupBytes = (size_t)96 << 20;
+
+bool batch_planar_method(const Method& mt) { return mt.P2 <= 255 && !(mt.flags & (4 | 8)); }
+
+int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& mt, cudaStream_t s,
+                     bool grow, int* launches) {
+  auto sums = [&](int i) {
+    return layout_for(probs[i].W, probs[i].H, probs[i].D, mt.wide != 0);
+  };
+  auto planes = [&](int i) {
+    return layout_single(probs[i].W, probs[i].H, probs[i].D, mt);
+  };
+  std::vector<Layout> lay((size_t)n);
+  size_t largest = 0;
+  for (int i = 0; i < n; i++) {
+    lay[i] = planes(i);
+    largest = std::max(largest, lay[i].total);
+  }
+  if (grow && largest > e->scratch_cap) {  // half of the device's memory stays free with it
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
+        largest + total_b / 2 <= free_b + e->scratch_cap) {
+      cudaDeviceSynchronize();  // a batch may still run in the old scratch
+      void* p = nullptr;
+      if (cudaMalloc(&p, largest) == cudaSuccess) {
+        cudaFree(e->scratch);
+        e->scratch = static_cast<char*>(p);
+        e->scratch_cap = largest;
+      }
+    }
+    cudaGetLastError();
+  }
+  for (int i = 0; i < n; i++)
+    if (lay[i].total > e->scratch_cap) lay[i] = sums(i);
+  // groups: pairs of one D and one setting, largest first
+  std::vector<int> order((size_t)n);
+  std::iota(order.begin(), order.end(), 0);
+  auto tune = [&](int i) -> const BatchTune& {
+    return e->tune[tune_bucket(probs[i].W, probs[i].H, probs[i].D)];
+  };
+  auto alike = [&](int a, int b) {
+    return probs[a].D == probs[b].D && lay[a].planes && lay[b].planes &&
+           tune(a).row_dpl == tune(b).row_dpl && tune(a).wta_px == tune(b).wta_px;
+  };
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+    if (probs[a].D != probs[b].D) return probs[a].D > probs[b].D;
+    return lay[a].total > lay[b].total;
+  });
+  struct Group {
+    int first, n;
+    size_t bytes;
+  };
+  std::vector<Group> groups;
+  const size_t most = std::min(kPlanarGroupBytes, e->scratch_cap);
+  for (int i = 0; i < n;) {
+    Group g{i, 1, lay[order[i]].total};
+    for (i++; i < n && g.n < kGroupPairs && alike(order[g.first], order[i]) &&
+              g.bytes + lay[order[i]].total <= most;
+         i++, g.n++)
+      g.bytes += lay[order[i]].total;
+    groups.push_back(g);
+  }
+  std::stable_sort(groups.begin(), groups.end(),
+                   [](const Group& a, const Group& b) { return a.bytes > b.bytes; });
+  // slots: group k runs in slot k % slots, whose part of the scratch holds its largest group
+  const int G = (int)groups.size();
+  int slots = 1;
+  size_t need = groups[0].bytes;
+  while (slots < kSlots && slots < G && need + groups[slots].bytes <= e->scratch_cap)
+    need += groups[slots++].bytes;
+  size_t base[kSlots] = {};
+  for (int k = 1; k < slots; k++) base[k] = base[k - 1] + groups[k - 1].bytes;
+  // a batch of this engine on another stream may still use the scratch (a capturing stream cannot
+  // wait for work outside its capture)
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t c = cudaStreamIsCapturing(s, &cap);
+  const bool capturing = cap != cudaStreamCaptureStatusNone;
+  if (c == cudaSuccess && !capturing) c = cudaStreamWaitEvent(s, e->ev_end, 0);
+  if (slots > 1 && c == cudaSuccess) {
+    c = cudaEventRecord(e->ev_start, s);
+    for (int k = 0; k < slots && c == cudaSuccess; k++)
+      c = cudaStreamWaitEvent(e->main[k], e->ev_start, 0);
+  }
+  int total = 0;
+  PairGroup pg;
+  for (int gi = 0; gi < G && c == cudaSuccess; gi++) {
+    const Group& g = groups[gi];
+    const int sl = gi % slots;
+    cudaStream_t st = slots > 1 ? e->main[sl] : s;
+    char* at = e->scratch + base[sl];
+    pg.n = g.n;
+    for (int i = 0; i < g.n; i++) {
+      const int k = order[g.first + i];
+      const Problem& q = probs[k];
+      Problem& pb = pg.p[i];
+      pb = problem_at(at, lay[k], q.W, q.H, q.D);
+      pb.left = q.left;
+      pb.right = q.right;
+      pb.in_pitch = q.in_pitch;
+      pb.disp = q.disp;
+      pb.out_pitch = q.out_pitch;
+      pb.dlf = nullptr;
+      at += lay[k].total;
+    }
+    if (pg.p[0].planar) {
+      const BatchTune& tn = tune(order[g.first]);
+      c = run_group(pg, mt, tn.row_dpl, tn.wta_px / 2, st);
+      total += 6;
+    } else {
+      int l = 0;
+      c = run_pipeline(pg.p[0], mt, default_tuning(pg.p[0].D), st, &l);
+      total += l;
+    }
+  }
+  if (slots > 1) {
+    for (int k = 0; k < slots && c == cudaSuccess; k++) {
+      c = cudaEventRecord(e->ev_join[k], e->main[k]);
+      if (c == cudaSuccess) c = cudaStreamWaitEvent(s, e->ev_join[k], 0);
+    }
+  }
+  if (c == cudaSuccess && !capturing) c = cudaEventRecord(e->ev_end, s);
+  if (c != cudaSuccess) return set_err(e, c, "batch launch");
+  if (launches) *launches = total;
   return 0;
 }
 

@@ -1,0 +1,80 @@
+"""Path planes (P2 <= 255): every lane count of the sheared chains, one plane per pair of opposite
+directions (2 P2 <= 255) and one per direction, against the oracle, bit by bit; and the batch route
+on them at its limits of group size and scratch."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2106_07927_gb300 import binding, scenes
+
+pytestmark = pytest.mark.gpu
+
+
+def _pair(seed, W, H, D):
+    left, right, _ = scenes.make_scene(("road", "nadir")[seed % 2], seed, W, H, D)
+    return left, right
+
+
+# D / 16 = 1 .. 16 lanes per chain, with the row path's 2, 4 and 8 disparities per lane; images
+# narrower than D, than a warp's chains and than two row chunks; P2 at the byte limits 127, 128, 255.
+@pytest.mark.parametrize("D", range(16, 257, 16))
+@pytest.mark.parametrize("W,H,p2,paths", [(61, 23, 127, 8), (40, 9, 128, 8), (9, 40, 255, 4),
+                                          (131, 6, 127, 4), (1, 5, 255, 8)])
+def test_planes_match_oracle(D, W, H, p2, paths):
+    import torch
+    rng = np.random.default_rng(D + W)
+    left = rng.integers(0, 256, (H, W)).astype(np.uint8)
+    right = np.roll(left, -3, axis=1)
+    prm = scenes.params(W, H, D, 9, 7, 11, p2, paths, 3)
+    ref, dbg = oracle.sgm(left, right, D, 9, 7, 11, p2, paths, 3, 1, debug=True)
+    st = binding.Stereo(prm)
+    L, R = torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda()
+    for dpl in (2, 4, 8):
+        if D // dpl > 32:
+            continue
+        binding.res2tac_set_tuning(st.handle, binding.res2tac_tuning(agg_dpl=dpl))
+        out = st.compute(L, R)
+        got = st.debug_outputs()
+        torch.cuda.synchronize()
+        assert np.array_equal(got["cost"].cpu().numpy(), dbg["cost"])
+        for k in ("agg", "dl", "dr"):
+            assert np.array_equal(binding.u16(got[k]), dbg[k]), (k, dpl)
+        assert np.array_equal(binding.u16(out), ref), dpl
+    st.close()
+
+
+@pytest.mark.parametrize("p2", [120, 200])
+def test_batch_groups_and_scratch_limits(p2):
+    import torch
+    # 40 pairs of one size (more than a group holds), two of another D, one large one
+    shapes = [(50, 30, 32)] * 40 + [(70, 20, 48)] * 2 + [(300, 200, 128)]
+    prm = scenes.params(64, 64, 64, 9, 7, 10, p2, 8, 3)
+    pairs, outs, want, keep = [], [], [], []
+    for i, (W, H, D) in enumerate(shapes):
+        left, right = _pair(i, W, H, D)
+        L, R = torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda()
+        o = torch.full((H, W), -1, dtype=torch.int16, device="cuda")
+        keep.append((L, R))
+        outs.append(o)
+        pairs.append(binding.res2tac_pair(L.data_ptr(), R.data_ptr(), W, o.data_ptr(), 2 * W, W, H,
+                                          D, 0))
+        want.append(oracle.sgm(left, right, D, 9, 7, 10, p2, 8, 3))
+    params = binding.params_from_dict(prm)
+    one = binding.res2tac_batch_workspace_bytes(params, pairs[-1:])
+    # grown on demand; reserved for the batch; reserved for less than the large pair's planes
+    for reserve, batch in ((0, pairs), (binding.res2tac_batch_workspace_bytes(params, pairs), pairs),
+                           (one, pairs[-1:])):
+        ctx = binding.Stereo(prm)
+        if reserve:
+            binding.res2tac_batch_reserve(ctx.handle, reserve, len(batch))
+        for o in outs:
+            o.fill_(-1)
+        # twice, on two streams: the second call uses the same scratch
+        s2 = torch.cuda.Stream()
+        s2.wait_stream(torch.cuda.current_stream())
+        binding.res2tac_compute_batch(ctx.handle, batch, torch.cuda.current_stream().cuda_stream)
+        binding.res2tac_compute_batch(ctx.handle, batch, s2.cuda_stream)
+        torch.cuda.synchronize()
+        for o, w in list(zip(outs, want))[-len(batch):]:
+            assert np.array_equal(binding.u16(o), w)
+        ctx.close()
