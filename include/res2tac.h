@@ -113,11 +113,13 @@ typedef struct res2tac_pair {
  * row_cost: costs of the row-path kernel: 1 = read from the cost volume, 2 = recomputed from the
  *   census descriptors inside the walk (popcount of the XOR per step; census cost with
  *   row_mode 2 and D = 32 agg_dpl only, other settings read the volume).
- * Automatic values: agg_dpl 2 for D <= 64, 4 for D <= 128, else 8; agg_warps 2; shear_dpl 16;
- * row_mode 2; cost_mode 1 (measured faster); row_cost 1; wta_chunk 64 and shear_cpl 1 for a context
- * on path planes (see res2tac_create), else wta_chunk 128 and shear_cpl 2 at D = 128, 1 otherwise.
- * A context on path planes uses them for calls with shear_dpl 16, row_mode 2, cost_mode 1 and
- * row_cost 1 (agg_warps has no effect there), and sums in place with any other setting. */
+ * Automatic values: agg_dpl 2 for D <= 64, 4 for D <= 128, else 8; agg_warps 2; row_mode 2;
+ * cost_mode 1 (measured faster); row_cost 1; for a context on path planes (see res2tac_create)
+ * wta_chunk 64, shear_cpl 1 and shear_dpl 8 on small images, else 16; otherwise wta_chunk 128,
+ * shear_dpl 16, shear_cpl 2 at D = 128, else 1.
+ * A context on path planes uses them for calls with shear_dpl 8 or 16, shear_cpl 1, row_mode 2,
+ * cost_mode 1 and row_cost 1 (agg_warps has no effect there), and adds its sums in place with any
+ * other setting. */
 typedef struct res2tac_tuning {
   int32_t agg_dpl;
   int32_t agg_warps;

@@ -101,6 +101,11 @@ struct res2tac_ctx {
   r2t::Fork fork;     // second stream for the concurrent aggregation kernels
 };
 
+// The automatic settings of a context.
+static r2t::Tuning auto_tuning(const res2tac_ctx* h) {
+  return h->lay.planes ? r2t::default_planar_tuning(h->p.width, h->p.max_disp, h->p.num_paths)
+                       : r2t::default_tuning(h->p.max_disp);
+}
 
 extern "C" {
 
@@ -150,7 +155,7 @@ int res2tac_create(const res2tac_params* p, res2tac_t* out) {
     h->scratch = nullptr;
   }
   if (!h->scratch) e = cudaMalloc(&h->scratch, h->lay.total);
-  h->tuning = r2t::default_tuning(p->max_disp, h->lay.planes != 0);
+  h->tuning = auto_tuning(h);
   if (e == cudaSuccess) e = cudaMemset(h->scratch + h->lay.fault, 0, 16);  // range-check record
   if (e == cudaSuccess) e = cudaMalloc(&h->stage_in, align_up(npx * 2, 256));
   if (e == cudaSuccess) e = cudaMalloc(&h->stage_out, align_up(npx * 2, 256));
@@ -410,7 +415,7 @@ int res2tac_get_tuning(res2tac_t h, res2tac_tuning* t) {
 
 int res2tac_set_tuning(res2tac_t h, const res2tac_tuning* t) {
   if (!h || !t) return fail(RES2TAC_EINVAL, "NULL argument");
-  r2t::Tuning n = r2t::default_tuning(h->p.max_disp, h->lay.planes != 0);
+  r2t::Tuning n = auto_tuning(h);
   if (t->agg_dpl) n.agg_dpl = t->agg_dpl;
   if (t->agg_warps) n.agg_warps = t->agg_warps;
   if (t->wta_chunk) n.wta_chunk = t->wta_chunk;

@@ -112,7 +112,7 @@ __global__ void agg_copy_kernel(const void* src, uint16_t* dst, int64_t n) {
   }
 }
 
-Tuning default_tuning(int D, bool planar) {
+Tuning default_tuning(int D) {
   Tuning t;
   t.agg_dpl = long_dpl_default(D);
   t.agg_warps = 2;  // two warps per block (measured best with one row direction per lane group)
@@ -122,12 +122,16 @@ Tuning default_tuning(int D, bool planar) {
   t.row_split = 1;  // one row direction per lane group (measured 2 % faster at D = 128)
   t.cost_mode = 0;  // population counts: measured faster than the tensor-core kernel
   t.row_cost = 0;   // the row kernel reads the cost volume
-  if (planar) {
-    // 1242 x 375, D = 128: 0.158 ms for the stage with one chain per lane, 0.173 with two;
-    // selection tiles of 64 pixels 0.051 ms, of 128 0.057 (1920 x 1080, D = 256: 0.455, 0.480)
-    t.shear_cpl = 1;
-    t.wta_chunk = 64;
-  }
+  return t;
+}
+
+Tuning default_planar_tuning(int W, int D, int num_paths) {
+  Tuning t = default_tuning(D);
+  t.shear_dpl = planar_shear_dpl(2 * planar_long_pairs(W, num_paths), W);
+  t.shear_cpl = 1;
+  // 1242 x 375, D = 128: tiles of 64 pixels 0.051 ms, of 128 0.057 (1920 x 1080, D = 256: 0.455,
+  // 0.480)
+  t.wta_chunk = 64;
   return t;
 }
 

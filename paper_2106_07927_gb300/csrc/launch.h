@@ -27,8 +27,9 @@ struct Fork {
 cudaError_t fork_create(Fork* f);
 void fork_destroy(Fork* f);
 
-// Default configuration for a disparity count D; planar: of the path-plane kernels.
-Tuning default_tuning(int D, bool planar = false);
+// Default configuration for a disparity count D, and of a pair on path planes.
+Tuning default_tuning(int D);
+Tuning default_planar_tuning(int W, int D, int num_paths);
 // True when the configuration can run a pair with D disparities.
 bool tuning_valid(const Tuning& t, int D);
 
@@ -65,10 +66,11 @@ inline cudaError_t launch_agg(void (*kernel)(P...), int grid, int threads, size_
   cfg.numAttrs = dependent ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
-// Settings the plane kernels have (blocks are always one pair of warps): 16 disparities per lane of the sheared chains, one row
-// direction per lane group, costs from the volume of the population-count kernel.
+// Settings the plane kernels have (blocks are always one pair of warps): 16 disparities and one chain
+// per lane of the sheared chains, or (8) one chain per warp, one row direction per lane group, costs from the
+// volume of the population-count kernel.
 inline bool planar_tuning(const Tuning& tn) {
-  return tn.shear_dpl == 16 && tn.row_split == 1 && tn.cost_mode == 0 && tn.row_cost == 0;
+  return (tn.shear_dpl == 8 || tn.shear_dpl == 16) && tn.shear_cpl == 1 && tn.row_split == 1 && tn.cost_mode == 0 && tn.row_cost == 0;
 }
 // Persistent batch variants of the two kernels, as handles for cudaLaunchKernel. Parameters:
 // (const BatchHeader*, const GroupDesc*, const Problem*, const AggSeg* segs,

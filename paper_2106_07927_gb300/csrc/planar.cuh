@@ -160,9 +160,54 @@ struct PairBytes<4> {
   }
 };
 
-// Rows y0 .. y0 + 32 / LPL - 1 in one direction, one per group of LPL lanes; lane member lig owns
-// words [lig NW, (lig + 1) NW). FULL: D == 2 NW LPL. ring: planar_row_smem(NW) bytes of this warp.
-// The two directions meet at pixel `mid` (a multiple of the chunk) when they share a plane.
+// Chains of one warp with few words per lane: groups of LPL lanes, lane member lig owns words
+// [lig NW, (lig + 1) NW). FULL: D == 2 NW LPL. The chain of one step, L -> neighbour shuffle -> L, is
+// its cost: the group minimum (one redux.sync when a chain takes the whole warp) runs beside it.
+template <int NW, int LPL, bool FULL>
+struct LongChain {
+  typedef PairBytes<NW> PB;
+  Ends ends;
+  bool owns;  // the lane holds words of its chain
+  uint32_t L[NW], mm;
+  __device__ __forceinline__ LongChain(int lane, int D)
+      : ends(lane, lane % LPL, FULL ? LPL : D / (2 * NW), FULL || lane % LPL < D / (2 * NW)),
+        owns(FULL || lane % LPL < D / (2 * NW)) {
+    restart();
+  }
+  // the next step starts a line of the path: L = C
+  __device__ __forceinline__ void restart() {
+#pragma unroll
+    for (int k = 0; k < NW; k++) L[k] = 0;
+    mm = 0;
+  }
+  // One step with the costs raw; returns the lane's bytes of U.
+  __device__ __forceinline__ typename PB::T step(typename PB::T raw, uint32_t P1P1,
+                                                 uint32_t P2P2) {
+    uint32_t cst[NW], U[NW], Ln[NW];
+    PB::unpack(raw, cst);
+    const uint32_t up = ends.prev(L[NW - 1]), dn = ends.next(L[0]);
+    const uint32_t mP2 = mm + P2P2;
+    uint32_t lmin = 0;
+#pragma unroll
+    for (int k = 0; k < NW; k++) {
+      const uint32_t t =
+          vmin2(k == 0 ? up : L[(k + NW - 1) % NW], k == NW - 1 ? dn : L[(k + 1) % NW]) + P1P1;
+      U[k] = vmin3(t, L[k], mP2) - mm;  // halves >= m(q): no borrow
+      Ln[k] = U[k] + cst[k];
+      lmin = k == 0 ? Ln[0] : vmin2(lmin, Ln[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < NW; k++) L[k] = Ln[k];
+    lmin = halves_min(lmin);
+    if (!FULL) lmin = owns ? lmin : 0xFFFFFFFFu;
+    mm = group_min<LPL>(lmin);
+    return PB::pack(U);
+  }
+};
+
+// Rows y0 .. y0 + 32 / LPL - 1 in one direction, one per group of LPL lanes. ring:
+// planar_row_smem(NW) bytes of this warp. The two directions meet at pixel `mid` (a multiple of the
+// chunk) when they share a plane.
 template <int NW, int LPL, bool FULL, bool BACK>
 __device__ __forceinline__ void planar_rows(const Problem& pb, const Method& mt, int y0,
                                             uint8_t* ring) {
@@ -170,10 +215,9 @@ __device__ __forceinline__ void planar_rows(const Problem& pb, const Method& mt,
   constexpr int CPW = 32 / LPL, G = kRowChunk;
   const int lane = threadIdx.x & 31, c = lane / LPL, lig = lane % LPL;
   const int W = pb.W, D = FULL ? 2 * NW * LPL : pb.D;
-  const int nl = FULL ? LPL : D / (2 * NW);
   const int y = y0 + c;
-  const bool valid = y < pb.H, active = valid && (FULL || lig < nl);
-  const Ends ends(lane, lig, nl, FULL || lig < nl);
+  LongChain<NW, LPL, FULL> chain(lane, D);
+  const bool valid = y < pb.H, active = valid && chain.owns;
   const bool paired = planar_paired(mt);
   const int64_t row = (int64_t)(valid ? y : 0) * W * D;
   const uint32_t slot_bytes = (uint32_t)(CPW * G * D);
@@ -186,9 +230,6 @@ __device__ __forceinline__ void planar_rows(const Problem& pb, const Method& mt,
   const int64_t nde = (int64_t)W * pb.H * D;  // extent of the volumes (range checks)
   (void)nde;
 
-  uint32_t L[NW], mm = 0;
-#pragma unroll
-  for (int k = 0; k < NW; k++) L[k] = 0;
   // pixels [q0, q1), walked from q1 - 1 down when BACK; add: onto the other direction's U
   auto walk = [&](int q0, int q1, auto add_) {
     constexpr bool add = decltype(add_)::value;
@@ -218,25 +259,7 @@ __device__ __forceinline__ void planar_rows(const Problem& pb, const Method& mt,
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
     auto step = [&](typename PB::T raw, typename PB::T oth, uint8_t* out) {
-      uint32_t cst[NW], U[NW], Ln[NW];
-      PB::unpack(raw, cst);
-      const uint32_t up = ends.prev(L[NW - 1]), dn = ends.next(L[0]);
-      const uint32_t mP2 = mm + P2P2;
-      uint32_t lmin = 0;
-#pragma unroll
-      for (int k = 0; k < NW; k++) {
-        const uint32_t t =
-            vmin2(k == 0 ? up : L[(k + NW - 1) % NW], k == NW - 1 ? dn : L[(k + 1) % NW]) + P1P1;
-        U[k] = vmin3(t, L[k], mP2) - mm;  // halves >= m(q): no borrow
-        Ln[k] = U[k] + cst[k];
-        lmin = k == 0 ? Ln[0] : vmin2(lmin, Ln[k]);
-      }
-#pragma unroll
-      for (int k = 0; k < NW; k++) L[k] = Ln[k];
-      lmin = halves_min(lmin);
-      if (!FULL) lmin = active ? lmin : 0xFFFFFFFFu;
-      mm = group_min<LPL>(lmin);
-      typename PB::T u = PB::pack(U);
+      typename PB::T u = chain.step(raw, P1P1, P2P2);
       if (add) PB::add(u, oth);  // bytes add without a carry
       if (active && R2T_CHECKED(pb, out, 2 * NW, pb.agg, planar_planes(mt) * nde, 2))
         PB::store(out, u);
@@ -286,19 +309,35 @@ __device__ __forceinline__ void planar_rows(const Problem& pb, const Method& mt,
 }
 
 // ------------------------------------------------------------------------------- sheared columns
-// The sheared chains of aggregate.cuh on planes: NL = D / 16 lanes per chain, 8 words (16
-// disparities, 16 bytes of each volume) per lane and chain, CPL chains per lane. Groups of any
-// number of lanes share a warp (D = 144: three chains of 9 lanes). A lane copies its own 16 cost
-// bytes of a step to shared memory 6 steps ahead and stores its own 16 bytes of U, so the lanes of
-// a warp never wait for each other's copies; adjacent chains sit on adjacent pixels, so both
-// are contiguous over the warp.
+// The sheared chains of aggregate.cuh on planes, in one of two shapes (planar_shear_dpl):
+// - planar_shear: NL = D / 16 lanes per chain, 8 words (16 disparities, 16 bytes of each volume) per
+//   lane; groups of any number of lanes share a warp (D = 144: three chains of 9 lanes). A lane
+//   copies its own 16 cost bytes of a step to shared memory 6 steps ahead and stores its own 16
+//   bytes of U, so the lanes of a warp never wait for each other's copies; adjacent chains sit on
+//   adjacent pixels, so both are contiguous over the warp. The fewest instructions per estimate.
+// - planar_long: one chain per warp, as the row paths. The shortest step, for small images.
 constexpr int kPlanarRing = 8;
-// (of one warp)
-__host__ __device__ inline int planar_shear_smem(int cpl) { return kPlanarRing * 1024 * cpl; }
-// Pairs of warps: the two opposite directions of a group of adjacent chains.
-__host__ __device__ inline int planar_shear_pairs(int W, int D, int num_paths, int cpl) {
-  const int ch = cpl * (32 / (D / 16));
+__host__ __device__ inline int planar_shear_smem() { return kPlanarRing * 1024; }  // of one warp
+// Pairs of warps: the two opposite directions of a group of adjacent chains, or of one chain.
+__host__ __device__ inline int planar_shear_pairs(int W, int D, int num_paths) {
+  const int ch = 32 / (D / 16);
   return shear_kinds(num_paths) / 2 * ((W + ch - 1) / ch);
+}
+__host__ __device__ inline int planar_long_pairs(int W, int num_paths) {
+  return shear_kinds(num_paths) / 2 * W;
+}
+// Words per lane of the one-chain-per-warp shape.
+__host__ __device__ inline int planar_long_words(int D) { return D <= 64 ? 1 : (D <= 128 ? 2 : 4); }
+// Shape of a launch over pairs of that many chains in all (setting shear_dpl): 8 for one chain per
+// warp, 16 otherwise. The line lies where the warps of the 16-disparity shape leave most schedulers
+// with one or none, so that a step's latency decides: us per call with one chain per warp and with
+// 16 disparities per lane, 8 paths: 160x120 D=32 (960 chains) 38, 44; 320x240 D=64 (1920) 54, 66;
+// 413x307 D=48 (2478) 83, 80; 640x480 D=64 (3840) 138, 132; 1242x375 D=128 (7452) 280, 262.
+// wmin: the smallest width among them (a chunk of the one-chain-per-warp walk wraps around the image
+// edge at most once).
+constexpr int64_t kLongChains = 2200;
+inline int planar_shear_dpl(int64_t chains, int wmin) {
+  return wmin >= kRowChunk && chains <= kLongChains ? 8 : 16;
 }
 
 // Minimum over the NL lanes of a group of a value whose halves are equal. Any NL: rotations by
@@ -342,21 +381,22 @@ struct GroupMin {
   }
 };
 
-// One direction (back: the upward one) of pair `item`: CH adjacent chains of one kind. Pairs of
-// steps in which no chain of the warp wraps around the image edge (nor its copies, 6 steps ahead)
-// and which are not among the last rows of the walk take the fast path; te is the first step of the
-// next pair that does not. Steps are counted from the start of each of the walk's two parts.
-template <int NL, int CPL>
+// One direction (back: the upward one) of pair `item`: adjacent chains of one kind. Groups of GS
+// steps in which no chain of the warp wraps around the image edge (nor its copies, PF steps ahead)
+// and which are not among the last rows of the walk take the fast path; te is the first step of
+// the next group that does not. Steps are counted from the start of each of the walk's two parts.
+template <int NL>
 __device__ __forceinline__ void planar_shear(const Problem& pb, const Method& mt, int item,
                                              bool back, uint8_t* ring) {
-  constexpr int NP = 8, D = 16 * NL, CPW = 32 / NL, CH = CPW * CPL, KS = kPlanarRing, PF = KS - 2;
-  constexpr int SLOT = 1024 * CPL, OTHER = 512 * CPL;  // costs, then the other direction's U
+  constexpr int NP = 8, LB = 16, D = LB * NL, CH = 32 / NL;
+  constexpr int GS = 2, KS = kPlanarRing, PF = KS - GS;
+  constexpr int SLOT = 1024, OTHER = 512;  // costs, then the other direction's U
   const int lane = threadIdx.x & 31, c = lane / NL, lig = lane - c * NL;
-  const bool in = c < CPW;
+  const bool in = c < CH;
   const int W = pb.W, H = pb.H;
   const int ng = (W + CH - 1) / CH;
   const int kp = item / ng;  // kinds 2 kp (down) and 2 kp + 1 (up)
-  const int j0 = (item - kp * ng) * CH;
+  const int j = (item - kp * ng) * CH + c;
   const int sh = kp == 0 ? 0 : (kp == 1 ? 1 : -1);
   const bool paired = planar_paired(mt);
   const int dy = back ? -1 : 1, dx = back ? -sh : sh;
@@ -364,7 +404,7 @@ __device__ __forceinline__ void planar_shear(const Problem& pb, const Method& mt
   const Ends ends(lane, lig, NL, in);
   const GroupMin<NL> gmin(lane, lig, in);
   const uint32_t P1P1 = (uint32_t)mt.P1 * 0x10001u, P2P2 = (uint32_t)mt.P2 * 0x10001u;
-  const uint32_t own = (uint32_t)__cvta_generic_to_shared(ring) + 16u * lane;
+  const uint32_t own = (uint32_t)__cvta_generic_to_shared(ring) + (uint32_t)(LB * lane);
   // offsets into a volume, modulo 2^32 (planar volumes are smaller, see layout.h)
   const uint32_t stride = (uint32_t)((dy * W + dx) * D);
   const uint32_t wrap = (uint32_t)(dx * W * D);  // taken off where a chain wraps around the edge
@@ -374,175 +414,261 @@ __device__ __forceinline__ void planar_shear(const Problem& pb, const Method& mt
   const uint8_t* const cost = pb.cost;
   uint8_t* const plane = reinterpret_cast<uint8_t*>(pb.agg) +
                          (int64_t)(paired ? 1 + kp : 2 + 2 * kp + (back ? 1 : 0)) * pb.plane;
-  bool act[CPL];
-  uint32_t ro[CPL], wo[CPL];  // offsets of the next cost copy and the next store
-  int tw[CPL], tr[CPL];       // steps at which the chain and its copies next wrap
-  uint32_t L[CPL][NP], mm[CPL];
+  const bool act = in && j < W;
+  int x = act ? (j + sh * ystart) % W : 0;
+  if (x < 0) x += W;
+  uint32_t wo = (uint32_t)(((int64_t)ystart * W + x) * D + LB * lig);  // offset of the next store
+  int tw = !act || dx == 0 ? kNever : (dx > 0 ? W - x : x + 1);  // step of the chain's next wrap
+  uint32_t L[NP], mm = 0;
 #pragma unroll
-  for (int g = 0; g < CPL; g++) {
-    const int j = j0 + c + CPW * g;
-    act[g] = in && j < W;
-    int x = act[g] ? (j + sh * ystart) % W : 0;
-    if (x < 0) x += W;
-    wo[g] = (uint32_t)(((int64_t)ystart * W + x) * D + 16 * lig);
-    tw[g] = !act[g] || dx == 0 ? kNever : (dx > 0 ? W - x : x + 1);
-#pragma unroll
-    for (int k = 0; k < NP; k++) L[g][k] = 0;
-    mm[g] = 0;
-  }
+  for (int k = 0; k < NP; k++) L[k] = 0;
   // n steps; add: onto the other direction's U
   auto walk = [&](int n, auto add_) {
     constexpr bool add = decltype(add_)::value;
-#pragma unroll
-    for (int g = 0; g < CPL; g++) {
-      ro[g] = wo[g];
-      tr[g] = tw[g];
-    }
-    auto fetch = [&](int g, uint32_t o, uint32_t slot) {
-      if (act[g] && R2T_CHECKED(pb, cost + o, 16, pb.cost, nde, 3))
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + 512 * g),
-                     "l"(cost + o)
+    uint32_t ro = wo;  // offset of the next cost copy, and the step of its next wrap
+    int tr = tw;
+    auto fetch = [&](uint32_t o, uint32_t slot) {
+      if (act && R2T_CHECKED(pb, cost + o, LB, pb.cost, nde, 3))
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot), "l"(cost + o)
                      : "memory");
-      if (add && act[g] && R2T_CHECKED(pb, plane + o, 16, pb.agg, planar_planes(mt) * nde, 3))
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + OTHER + 512 * g),
+      if (add && act && R2T_CHECKED(pb, plane + o, LB, pb.agg, planar_planes(mt) * nde, 3))
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + OTHER),
                      "l"(plane + o)
                      : "memory");
     };
     auto copy_step = [&](int t) {  // any step (past the last one: nothing)
       if (t < n) {
-        const uint32_t slot = own + (uint32_t)((t & (KS - 1)) * SLOT);
-#pragma unroll
-        for (int g = 0; g < CPL; g++) {
-          if (tr[g] == t) {
-            ro[g] -= wrap;
-            tr[g] += W;
-          }
-          fetch(g, ro[g], slot);
-          ro[g] += stride;
+        if (tr == t) {
+          ro -= wrap;
+          tr += W;
         }
+        fetch(ro, own + (uint32_t)((t & (KS - 1)) * SLOT));
+        ro += stride;
       }
     };
-    // one step from the values La to Lb (two steps of the loop return to the same registers)
-    auto step = [&](uint32_t slot, const uint32_t (&o)[CPL], const uint32_t (&La)[CPL][NP],
-                    uint32_t (&Lb)[CPL][NP]) {
-      uint4 raw[CPL], oth[CPL];
-#pragma unroll
-      for (int g = 0; g < CPL; g++) {
-        raw[g] = lds128(slot + 512 * g);
-        if (add) oth[g] = lds128(slot + OTHER + 512 * g);
-      }
-      uint32_t up[CPL], dn[CPL], mP2[CPL], lm[CPL], u[CPL][4];
-#pragma unroll
-      for (int g = 0; g < CPL; g++) {
-        up[g] = ends.prev(La[g][NP - 1]);
-        dn[g] = ends.next(La[g][0]);
-        mP2[g] = mm[g] + P2P2;
-      }
+    // one step from the values La to Lb (a group's steps return to the same registers)
+    auto step = [&](uint32_t slot, uint32_t o, const uint32_t (&La)[NP], uint32_t (&Lb)[NP]) {
+      const uint4 raw = lds128(slot);
+      uint4 oth = make_uint4(0, 0, 0, 0);
+      if (add) oth = lds128(slot + OTHER);
+      const uint32_t rw[4] = {raw.x, raw.y, raw.z, raw.w}, ow[4] = {oth.x, oth.y, oth.z, oth.w};
+      const uint32_t up = ends.prev(La[NP - 1]), dn = ends.next(La[0]);
+      const uint32_t mP2 = mm + P2P2;
+      uint32_t lm = 0, u[4];
 #pragma unroll
       for (int k = 0; k < NP; k += 2) {
-#pragma unroll
-        for (int g = 0; g < CPL; g++) {
-          uint32_t c0, c1;
-          unpack4(k == 0 ? raw[g].x : k == 2 ? raw[g].y : k == 4 ? raw[g].z : raw[g].w, c0, c1);
-          const uint32_t t0 = vmin2(k == 0 ? up[g] : La[g][(k + NP - 1) % NP], La[g][k + 1]) + P1P1;
-          const uint32_t t1 = vmin2(La[g][k], k + 2 < NP ? La[g][(k + 2) % NP] : dn[g]) + P1P1;
-          const uint32_t u0 = vmin3(t0, La[g][k], mP2[g]) - mm[g];  // halves >= m(q): no borrow
-          const uint32_t u1 = vmin3(t1, La[g][k + 1], mP2[g]) - mm[g];
-          Lb[g][k] = u0 + c0;
-          Lb[g][k + 1] = u1 + c1;
-          lm[g] = k == 0 ? vmin2(Lb[g][0], Lb[g][1]) : vmin3(lm[g], Lb[g][k], Lb[g][k + 1]);
-          u[g][k / 2] = __byte_perm(u0, u1, 0x6420);
-        }
+        uint32_t c0, c1;
+        unpack4(rw[k / 2], c0, c1);
+        const uint32_t t0 = vmin2(k == 0 ? up : La[(k + NP - 1) % NP], La[k + 1]) + P1P1;
+        const uint32_t t1 = vmin2(La[k], k + 2 < NP ? La[(k + 2) % NP] : dn) + P1P1;
+        const uint32_t u0 = vmin3(t0, La[k], mP2) - mm;  // halves >= m(q): no borrow
+        const uint32_t u1 = vmin3(t1, La[k + 1], mP2) - mm;
+        Lb[k] = u0 + c0;
+        Lb[k + 1] = u1 + c1;
+        lm = k == 0 ? vmin2(Lb[0], Lb[1]) : vmin3(lm, Lb[k], Lb[k + 1]);
+        u[k / 2] = __byte_perm(u0, u1, 0x6420);
+        if (add) u[k / 2] += ow[k / 2];  // bytes add without a carry
       }
-#pragma unroll
-      for (int g = 0; g < CPL; g++) {
-        if (add) {  // bytes add without a carry
-          u[g][0] += oth[g].x;
-          u[g][1] += oth[g].y;
-          u[g][2] += oth[g].z;
-          u[g][3] += oth[g].w;
-        }
-        if (act[g] && R2T_CHECKED(pb, plane + o[g], 16, pb.agg, planar_planes(mt) * nde, 4))
-        {
-          const uint4 v = make_uint4(u[g][0], u[g][1], u[g][2], u[g][3]);
-          // bytes that this kernel does not read again leave the L2 first
-          if (add || !paired)
-            __stcs(reinterpret_cast<uint4*>(plane + o[g]), v);
-          else
-            *reinterpret_cast<uint4*>(plane + o[g]) = v;
-        }
-        mm[g] = gmin(halves_min(lm[g]));
+      if (act && R2T_CHECKED(pb, plane + o, LB, pb.agg, planar_planes(mt) * nde, 4)) {
+        const uint4 v = make_uint4(u[0], u[1], u[2], u[3]);
+        // bytes that this kernel does not read again leave the L2 first
+        if (add || !paired)
+          __stcs(reinterpret_cast<uint4*>(plane + o), v);
+        else
+          *reinterpret_cast<uint4*>(plane + o) = v;
       }
+      mm = gmin(halves_min(lm));
     };
-    // first step of the next pair with an event, from even step t on
-    const int tail = n <= PF + 1 ? 0 : (n - PF) & ~1;  // pairs whose copies reach past the end
+    // first step of the next group with an event, from a group's first step t on
+    const int tail = n < PF + GS ? 0 : (n - PF) & ~(GS - 1);  // its copies reach past the end
     auto next_event = [&](int t) {
-      int e = kNever;
-#pragma unroll
-      for (int g = 0; g < CPL; g++) e = min(e, min(tw[g], tr[g] - PF));
-      e = (int)__reduce_min_sync(0xffffffffu, (unsigned)max(e, 0)) & ~1;
+      const int e =
+          (int)__reduce_min_sync(0xffffffffu, (unsigned)max(min(tw, tr - PF), 0)) & ~(GS - 1);
       return max(min(e, tail), t);
     };
 
 #pragma unroll
-    for (int s = 0; s < PF; s += 2) {
+    for (int s = 0; s < PF; s++) {
       copy_step(s);
-      copy_step(s + 1);
-      asm volatile("cp.async.commit_group;" ::: "memory");
+      if (s % GS == GS - 1) asm volatile("cp.async.commit_group;" ::: "memory");
     }
     int te = next_event(0);
     uint32_t rs = 0;  // ring offset of step t
-    for (int t = 0; t < n; t += 2) {
-      uint32_t o[CPL];
+    for (int t = 0; t < n; t += GS) {
       const uint32_t slot = own + rs, ahead = own + ((rs + PF * SLOT) & (KS * SLOT - 1));
-      rs = (rs + 2 * SLOT) & (KS * SLOT - 1);
+      rs = (rs + GS * SLOT) & (KS * SLOT - 1);
+      uint32_t M[NP];
       if (t < te) {
-#pragma unroll
-        for (int g = 0; g < CPL; g++) {
-          fetch(g, ro[g], ahead);
-          fetch(g, ro[g] + stride, ahead + SLOT);
-          ro[g] += 2 * stride;
-        }
+        fetch(ro, ahead);
+        fetch(ro + stride, ahead + SLOT);
+        ro += GS * stride;
         asm volatile("cp.async.commit_group;" ::: "memory");
         asm volatile("cp.async.wait_group 3;" ::: "memory");
-        uint32_t M[CPL][NP];
         step(slot, wo, L, M);
-#pragma unroll
-        for (int g = 0; g < CPL; g++) o[g] = wo[g] + stride;
-        step(slot + SLOT, o, M, L);
-#pragma unroll
-        for (int g = 0; g < CPL; g++) wo[g] += 2 * stride;
+        step(slot + SLOT, wo + stride, M, L);
+        wo += GS * stride;
       } else {
-        copy_step(t + PF);
-        copy_step(t + PF + 1);
+#pragma unroll
+        for (int u = 0; u < GS; u++) copy_step(t + PF + u);
         asm volatile("cp.async.commit_group;" ::: "memory");
         asm volatile("cp.async.wait_group 3;" ::: "memory");
-        for (int u = 0; u < 2 && t + u < n; u++) {
+        for (int u = 0; u < GS && t + u < n; u++) {
+          if (tw == t + u) {  // a new line of the path enters: L = C
 #pragma unroll
-          for (int g = 0; g < CPL; g++) {
-            if (tw[g] == t + u) {  // a new line of the path enters: L = C
-#pragma unroll
-              for (int k = 0; k < NP; k++) L[g][k] = 0;
-              mm[g] = 0;
-              wo[g] -= wrap;
-              tw[g] += W;
-            }
+            for (int k = 0; k < NP; k++) L[k] = 0;
+            mm = 0;
+            wo -= wrap;
+            tw += W;
           }
-          uint32_t M[CPL][NP];
           step(slot + (uint32_t)(u * SLOT), wo, L, M);
 #pragma unroll
-          for (int g = 0; g < CPL; g++)
-#pragma unroll
-            for (int k = 0; k < NP; k++) L[g][k] = M[g][k];
-#pragma unroll
-          for (int g = 0; g < CPL; g++) wo[g] += stride;
+          for (int k = 0; k < NP; k++) L[k] = M[k];
+          wo += stride;
         }
-        te = next_event(t + 2);
+        te = next_event(t + GS);
       }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
+    tw -= tw == kNever ? 0 : n;
+  };
+  if (paired) {
+    const int n0 = back ? H - H / 2 : H / 2;  // the two directions meet in the middle
+    walk(n0, std::false_type());
+    __syncthreads();
+    walk(H - n0, std::true_type());
+  } else {
+    walk(H, std::false_type());
+  }
+}
+
+// One direction of sheared chain `item` (all chains of kind pair 0, then of 1 and 2), the whole warp
+// on one chain. Costs are copied kRowChunk steps at a time, three chunks ahead, each lane the same
+// 16-byte pieces of every chunk. W >= kRowChunk. ring: planar_row_smem(NW) bytes of this warp.
+template <int NW, bool FULL>
+__device__ __forceinline__ void planar_long(const Problem& pb, const Method& mt, int item,
+                                            bool back, uint8_t* ring) {
+  typedef PairBytes<NW> PB;
+  constexpr int G = kRowChunk;
+  const int lane = threadIdx.x & 31;
+  const int W = pb.W, H = pb.H, D = FULL ? 64 * NW : pb.D;
+  const int kp = item / W;  // kinds 2 kp (down) and 2 kp + 1 (up)
+  const int j = item - kp * W;
+  const int sh = kp == 0 ? 0 : (kp == 1 ? 1 : -1);
+  const bool paired = planar_paired(mt);
+  const int dy = back ? -1 : 1, dx = back ? -sh : sh;
+  const int ystart = back ? H - 1 : 0;
+  LongChain<NW, 32, FULL> chain(lane, D);
+  const uint32_t P1P1 = (uint32_t)mt.P1 * 0x10001u, P2P2 = (uint32_t)mt.P2 * 0x10001u;
+  const uint32_t slot_bytes = (uint32_t)(G * D);
+  const uint32_t other = kRowStages * slot_bytes;  // the other direction's U behind the costs
+  const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
+  // offsets into a volume, modulo 2^32 (planar volumes are smaller, see layout.h)
+  const uint32_t stride = (uint32_t)((dy * W + dx) * D);
+  const uint32_t wrap = (uint32_t)(dx * W * D);  // taken off where the chain wraps around the edge
+  const int64_t nde = (int64_t)W * H * D;        // extent of the volumes (range checks)
+  (void)nde;
+  const uint8_t* const cost = pb.cost;
+  uint8_t* const plane = reinterpret_cast<uint8_t*>(pb.agg) +
+                         (int64_t)(paired ? 1 + kp : 2 + 2 * kp + (back ? 1 : 0)) * pb.plane;
+  const int ppx = D / 16;  // 16-byte pieces of a pixel; G ppx <= 32 NW of a chunk
+  int pu[NW], pq[NW];      // the lane's pieces: step in the chunk, piece of the pixel
 #pragma unroll
-    for (int g = 0; g < CPL; g++) tw[g] -= tw[g] == kNever ? 0 : n;
+  for (int v = 0; v < NW; v++) {
+    pu[v] = (lane + 32 * v) / ppx;
+    pq[v] = (lane + 32 * v) - pu[v] * ppx;
+  }
+  int x = (j + sh * ystart) % W;  // column of the next step
+  if (x < 0) x += W;
+  uint32_t wo = (uint32_t)(((int64_t)ystart * W + x) * D);  // and its offset
+  auto wrapped = [&](int& xx, uint32_t& o) {  // xx in (-W, 2 W)
+    if (xx >= W || xx < 0) {
+      xx -= dx * W;
+      o -= wrap;
+    }
+  };
+  bool fresh = false;  // the next step starts a line
+  // n steps; add: onto the other direction's U
+  auto walk = [&](int n, auto add_) {
+    constexpr bool add = decltype(add_)::value;
+    const int nch = (n + G - 1) / G;
+    int px[NW];  // column and offset of the lane's pieces of the next chunk to copy
+    uint32_t po[NW];
+#pragma unroll
+    for (int v = 0; v < NW; v++) {
+      px[v] = x + dx * pu[v];
+      po[v] = wo + pu[v] * stride;
+      wrapped(px[v], po[v]);
+      po[v] += 16 * pq[v];
+    }
+    auto copy = [&](int k) {
+      const uint32_t dst = ring_s + (uint32_t)(k & (kRowStages - 1)) * slot_bytes;
+#pragma unroll
+      for (int v = 0; v < NW; v++) {
+        if (pu[v] < G && k * G + pu[v] < n) {
+          const uint32_t a = dst + 16 * (lane + 32 * v), o = po[v];
+          if (R2T_CHECKED(pb, cost + o, 16, pb.cost, nde, 3))
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(cost + o)
+                         : "memory");
+          if (add && R2T_CHECKED(pb, plane + o, 16, pb.agg, planar_planes(mt) * nde, 3))
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a + other),
+                         "l"(plane + o)
+                         : "memory");
+        }
+        px[v] += G * dx;
+        po[v] += G * stride;
+        wrapped(px[v], po[v]);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto step = [&](typename PB::T raw, typename PB::T oth, uint32_t o) {
+      typename PB::T u = chain.step(raw, P1P1, P2P2);
+      if (add) PB::add(u, oth);  // bytes add without a carry
+      uint8_t* const out = plane + o + lane * 2 * NW;
+      if (chain.owns && R2T_CHECKED(pb, out, 2 * NW, pb.agg, planar_planes(mt) * nde, 4))
+        PB::store(out, u);
+    };
+#pragma unroll
+    for (int k = 0; k < kRowStages - 1; k++) copy(k);
+    for (int k = 0; k < nch; k++) {
+      __syncwarp();  // every lane is done with the slot refilled below
+      copy(k + kRowStages - 1);
+      asm volatile("cp.async.wait_group 3;" ::: "memory");
+      __syncwarp();
+      const uint32_t slot = ring_s + (uint32_t)(k & (kRowStages - 1)) * slot_bytes +
+                            (uint32_t)(lane * 2 * NW);
+      const int m = min(G, n - k * G);
+      const int last = x + G * dx;
+      if (m == G && !fresh && last < W && last >= 0) {  // no line starts in or after the chunk
+        typename PB::T raw[G], oth[G];
+#pragma unroll
+        for (int u = 0; u < G; u++) raw[u] = PB::load(slot + u * D);
+#pragma unroll
+        for (int u = 0; u < G; u++) {
+          oth[u] = typename PB::T();
+          if (add) oth[u] = PB::load(slot + other + u * D);
+        }
+#pragma unroll
+        for (int u = 0; u < G; u++) {
+          step(raw[u], oth[u], wo);
+          wo += stride;
+        }
+        x = last;
+      } else {
+        for (int u = 0; u < m; u++) {
+          if (fresh) chain.restart();
+          const uint32_t a = slot + u * D;
+          typename PB::T oth = typename PB::T();
+          if (add) oth = PB::load(a + other);
+          step(PB::load(a), oth, wo);
+          wo += stride;
+          x += dx;
+          fresh = x >= W || x < 0;
+          wrapped(x, wo);
+        }
+      }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
   };
   if (paired) {
     const int n0 = back ? H - H / 2 : H / 2;  // the two directions meet in the middle

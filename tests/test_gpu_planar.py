@@ -29,10 +29,10 @@ def test_planes_match_oracle(D, W, H, p2, paths):
     ref, dbg = oracle.sgm(left, right, D, 9, 7, 11, p2, paths, 3, 1, debug=True)
     st = binding.Stereo(prm)
     L, R = torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda()
-    for dpl in (2, 4, 8):
+    for dpl, sdpl in ((2, 16), (4, 8), (8, 16), (8, 8)):  # 8: one sheared chain per warp
         if D // dpl > 32:
             continue
-        binding.res2tac_set_tuning(st.handle, binding.res2tac_tuning(agg_dpl=dpl))
+        binding.res2tac_set_tuning(st.handle, binding.res2tac_tuning(agg_dpl=dpl, shear_dpl=sdpl))
         out = st.compute(L, R)
         got = st.debug_outputs()
         torch.cuda.synchronize()

@@ -6,13 +6,13 @@ import itertools
 import pytest
 
 NEVER = 1 << 30
-PF = 6  # steps between a cost copy and its use
 
 
 def _walk(W, H, kind, j, paired):
     """(copies, stores, restarts) of one chain alone in its warp, pixel by pixel, as the kernel's
-    two pointers and its fast and general pairs of steps make them, in one part or (directions
+    two pointers and its fast and general groups of GS steps make them, in one part or (directions
     that share a plane) in two; copies are listed by the step that uses them."""
+    GS, PF = 2, 6  # steps of a group, and between a cost copy and its use
     sh = 0 if kind < 2 else (1 if kind < 4 else -1)
     back = kind & 1
     dy, dx = (-1, -sh) if back else (1, sh)
@@ -26,7 +26,7 @@ def _walk(W, H, kind, j, paired):
     for ph in range(2 if paired else 1):
         n = H if not paired else (H // 2 if (ph == 0) != bool(back) else H - H // 2)
         rp, tr = wp, tw
-        tail = 0 if n <= PF + 1 else (n - PF) & ~1
+        tail = 0 if n < PF + GS else (n - PF) & ~(GS - 1)
 
         def copy_step(t):
             nonlocal rp, tr
@@ -38,7 +38,7 @@ def _walk(W, H, kind, j, paired):
                 rp += stride
 
         def next_event(t):
-            return max(min(max(min(tw, tr - PF), 0) & ~1, tail), t)
+            return max(min(max(min(tw, tr - PF), 0) & ~(GS - 1), tail), t)
 
         for s in range(PF):
             copy_step(s)
@@ -46,15 +46,16 @@ def _walk(W, H, kind, j, paired):
         t = 0
         while t < n:
             if t < te:
-                assert t + PF + 1 < n
-                copies += [rp, rp + stride]
-                rp += 2 * stride
-                stores += [wp, wp + stride]
-                wp += 2 * stride
+                assert t + PF + GS - 1 < n
+                for _ in range(GS):
+                    copies.append(rp)
+                    rp += stride
+                    stores.append(wp)
+                    wp += stride
             else:
-                copy_step(t + PF)
-                copy_step(t + PF + 1)
-                for u in range(2):
+                for u in range(GS):
+                    copy_step(t + PF + u)
+                for u in range(GS):
                     if t + u < n:
                         if tw == t + u:
                             restarts.append(base + t + u)
@@ -62,9 +63,50 @@ def _walk(W, H, kind, j, paired):
                             tw += W
                         stores.append(wp)
                         wp += stride
-                te = next_event(t + 2)
-            t += 2
+                te = next_event(t + GS)
+            t += GS
         tw -= 0 if tw == NEVER else n
+        base += n
+    return copies, stores, restarts
+
+
+def _long_walk(W, H, kind, j, paired):
+    """The same of the walk with one chain per warp: 8-step chunks, one cursor per step of a chunk."""
+    G = 8
+    sh = 0 if kind < 2 else (1 if kind < 4 else -1)
+    back = kind & 1
+    dy, dx = (-1, -sh) if back else (1, sh)
+    ystart = H - 1 if back else 0
+    x = (j + sh * ystart) % W
+    stride, wrap = dy * W + dx, dx * W
+    wo = ystart * W + x
+
+    def wrapped(xx, o):
+        return (xx - dx * W, o - wrap) if xx >= W or xx < 0 else (xx, o)
+
+    copies, stores, restarts = [], [], []
+    fresh, base = False, 0
+    for ph in range(2 if paired else 1):
+        n = H if not paired else (H // 2 if (ph == 0) != bool(back) else H - H // 2)
+        cur = [wrapped(x + dx * u, wo + u * stride) for u in range(G)]
+        for k in range((n + G - 1) // G):
+            for u in range(G):
+                if k * G + u < n:
+                    copies.append(cur[u][1])
+                cur[u] = wrapped(cur[u][0] + G * dx, cur[u][1] + G * stride)
+        for k in range((n + G - 1) // G):
+            m, last = min(G, n - k * G), x + G * dx
+            if m == G and not fresh and 0 <= last < W:
+                stores += [wo + u * stride for u in range(G)]
+                wo, x = wo + G * stride, last
+            else:
+                for u in range(m):
+                    if fresh:
+                        restarts.append(base + k * G + u)
+                    stores.append(wo)
+                    wo, x = wo + stride, x + dx
+                    fresh = x >= W or x < 0
+                    x, wo = wrapped(x, wo)
         base += n
     return copies, stores, restarts
 
@@ -81,6 +123,9 @@ def test_sheared_walk_on_planes(kind):
             for paired in (False, True):
                 got = _walk(W, H, kind, j, paired)
                 assert got == (want, want, starts), (W, H, j, paired)
+                if W >= 8:
+                    got = _long_walk(W, H, kind, j, paired)
+                    assert got == (want, want, starts), (W, H, j, paired, "long")
 
 
 @pytest.mark.parametrize("back", [False, True])
