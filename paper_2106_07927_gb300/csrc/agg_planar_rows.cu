@@ -7,7 +7,10 @@ namespace r2t {
 template <int NW, int LPL, bool FULL, class Src>
 __global__ void __launch_bounds__(kPairThreads)
     planar_row_kernel(const __grid_constant__ Src src, Method mt) {
-  launch_dependents();  // the sheared kernel's blocks follow as soon as every block here runs
+  // the sheared kernel's blocks follow as soon as every block here is past this wait, so what precedes
+  // this kernel is complete for them too
+  wait_prerequisites();
+  launch_dependents();
   extern __shared__ __align__(16) uint8_t shm[];
   int item = blockIdx.x;
   const Problem pb = src.locate(item);
@@ -23,7 +26,7 @@ template <int NW, int LPL, class Src>
 static cudaError_t launch_t(const Src& src, int D, int grid, const Method& mt, cudaStream_t s) {
   return launch_agg(D == 2 * NW * LPL ? planar_row_kernel<NW, LPL, true, Src>
                                       : planar_row_kernel<NW, LPL, false, Src>,
-                    grid, kPairThreads, 2 * planar_row_smem(NW), s, false, src, mt);
+                    grid, kPairThreads, 2 * planar_row_smem(NW), s, std::is_same<Src, OnePair>::value, src, mt);
 }
 
 template <class Src>

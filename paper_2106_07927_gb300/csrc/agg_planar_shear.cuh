@@ -16,6 +16,7 @@ __global__ void __launch_bounds__(kPairThreads)
   planar_shear<NL>(pb, mt, item, back, shm + (back ? planar_shear_smem() : 0));
   // this kernel starts beside the row kernel (after what precedes that one): it is complete only
   // when both are
+  launch_dependents();
   wait_prerequisites();
 }
 
@@ -27,6 +28,7 @@ __global__ void __launch_bounds__(kPairThreads)
   int item = blockIdx.x;
   const Problem pb = src.locate(item);
   planar_long<NW, FULL>(pb, mt, item, back, shm + (back ? planar_row_smem(NW) : 0));
+  launch_dependents();
   wait_prerequisites();
 }
 

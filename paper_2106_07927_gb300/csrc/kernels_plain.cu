@@ -12,6 +12,7 @@
 namespace r2t {
 
 __global__ void __launch_bounds__(256) census_kernel(Problem pb, Method mt) {
+  launch_dependents();
   __shared__ CensusSmem sm;
   census_tile_dispatch(pb, mt, blockIdx.x, sm);
 }
@@ -22,15 +23,19 @@ __global__ void __launch_bounds__(256) cost_kernel(Problem pb, Method mt) {
 }
 
 __global__ void __launch_bounds__(256) cost_planar_kernel(Problem pb, Method mt) {
+  wait_prerequisites();
   __shared__ CostSmem sm;
   if (mt.cw == 9)
     cost_tile_planar<true>(pb, blockIdx.x, sm);
   else
     cost_tile_planar<false>(pb, blockIdx.x, sm);
+  launch_dependents();
 }
 
 template <int R>
 __global__ void __launch_bounds__(256) wta_planar_kernel(Problem pb, int paths, int T) {
+  wait_prerequisites();
+  launch_dependents();
   extern __shared__ __align__(16) uint8_t wsm[];
   planar_wta_tile<R>(pb, paths, blockIdx.x, wsm, T);
 }
@@ -43,6 +48,7 @@ __global__ void __launch_bounds__(256) wta_dr_staged_kernel(Problem pb, int T) {
 
 template <bool SUB, bool WIDE>
 __global__ void __launch_bounds__(256) lr_median_kernel(Problem pb, Method mt) {
+  wait_prerequisites();
   __shared__ MedianSmemT<SUB> sm;
   lr_median_tile<SUB, WIDE>(pb, mt, blockIdx.x, sm);
 }
@@ -204,8 +210,8 @@ static cudaError_t launch_planar_wta_t(const Problem& pb, int paths, int T, cuda
   const size_t smem = planar_wta_smem(pb.D, T);
   cudaFuncSetAttribute(wta_planar_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)smem);
-  wta_planar_kernel<R><<<wta_items(pb.W, pb.H, T), 256, smem, s>>>(pb, paths, T);
-  return cudaGetLastError();
+  return launch_dep(wta_planar_kernel<R>, wta_items(pb.W, pb.H, T), 256, smem, s, pb, paths,
+                    T);
 }
 
 static cudaError_t launch_planar_wta(const Problem& pb, const Method& mt, const Tuning& tn,
@@ -233,7 +239,8 @@ static cudaError_t run_pass(const Problem& pb, const Method& mt, const Tuning& t
   } else {
     census_kernel<<<2 * census_items(pb.W, pb.H), 256, 0, s>>>(pb, mt);
     if (pb.planar) {
-      cost_planar_kernel<<<cost_items(pb.W, pb.H), 256, 0, s>>>(pb, mt);
+      e = launch_dep(cost_planar_kernel, cost_items(pb.W, pb.H), 256, 0, s, pb, mt);
+      if (e != cudaSuccess) return e;
     } else if (tn.cost_mode == 1 && cost_mma_ok(pb, mt)) {
       if ((e = launch_cost_mma(pb, mt, s)) != cudaSuccess) return e;
     } else {
@@ -320,15 +327,13 @@ cudaError_t run_pipeline(const Problem& pb, const Method& mt, const Tuning& tn, 
     return e;
   const int nm = median_items(pb.W, pb.H);
   nvtxRangePushA("res2tac lr check + median");
-  if (pb.disp_f == nullptr)  // uint16 map
-    lr_median_kernel<false, false><<<nm, 256, 0, s>>>(pb, mt);
-  else if (mt.wide)          // sub-pixel float map
-    lr_median_kernel<true, true><<<nm, 256, 0, s>>>(pb, mt);
-  else
-    lr_median_kernel<true, false><<<nm, 256, 0, s>>>(pb, mt);
+  e = launch_dep(pb.disp_f == nullptr ? lr_median_kernel<false, false>   // uint16 map
+                 : mt.wide            ? lr_median_kernel<true, true>     // sub-pixel float map
+                                      : lr_median_kernel<true, false>,
+                 nm, 256, 0, s, pb, mt);
   nvtxRangePop();
   n++;
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[exact ? 7 : 4], s);
   if (launches) *launches = n;
   return cudaSuccess;

@@ -44,11 +44,29 @@ cudaError_t launch_planar_rows(const Problem& pb, const Method& mt, const Tuning
                                cudaStream_t s);
 cudaError_t launch_planar_shear(const Problem& pb, const Method& mt, const Tuning& tn,
                                 cudaStream_t s);
-// Launches a kernel of the aggregation with the SM's memory split for the most shared memory: a
-// block is placed beside blocks of another kernel only when both ask for the same split. With the
-// driver's own choice the sheared kernel's blocks waited for the row kernel's to leave (1242 x
-// 375, D = 128: started at 75 us, on 118 of the SMs). dependent: may start its blocks as soon as
-// every block of the kernel before it has called launch_dependents.
+// Programmatic dependent launch: the kernel may start its blocks as soon as every block of the kernel
+// before it in the stream has called launch_dependents or ended; it waits by itself
+// (wait_prerequisites) before it touches memory.
+template <class... P, class... A>
+inline cudaError_t launch_dep(void (*kernel)(P...), int grid, int threads, size_t smem,
+                              cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+// An aggregation kernel, with the SM's memory split for the most shared memory: a block is placed
+// beside blocks of another kernel only when both ask for the same split. With the driver's own
+// choice the sheared kernel's blocks waited for the row kernel's to leave (1242 x 375, D = 128:
+// started at 75 us, on 118 of the SMs). The other stages keep the driver's choice (all on the same
+// split: 267 instead of 257 us a call).
 template <class... P, class... A>
 inline cudaError_t launch_agg(void (*kernel)(P...), int grid, int threads, size_t smem,
                               cudaStream_t s, bool dependent, A... args) {

@@ -70,15 +70,6 @@ struct Ends {
 // which left 4 blocks to an SM.)
 constexpr int kPairThreads = 64;
 
-// Programmatic dependent launch: lets the next kernel of the stream start its blocks / waits until
-// the kernel before this one is complete and its stores are visible.
-__device__ __forceinline__ void launch_dependents() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ void wait_prerequisites() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
 // Two opposite directions share a plane.
 __host__ __device__ inline bool planar_paired(const Method& mt) { return 2 * mt.P2 <= 255; }
 __host__ __device__ inline int planar_planes(const Method& mt) {
