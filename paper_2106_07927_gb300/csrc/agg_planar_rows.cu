@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(kPairThreads)
   const Problem pb = src.locate(item);
   const int y0 = item * (32 / LPL);
   if (threadIdx.x >= 32)
-    planar_rows<NW, LPL, FULL, true>(pb, mt, y0, shm + planar_row_smem(NW));
+    planar_rows<NW, LPL, FULL, true>(pb, mt, y0, shm + planar_ring_smem(pb.D, LPL));
   else
     planar_rows<NW, LPL, FULL, false>(pb, mt, y0, shm);
 }
@@ -26,7 +26,7 @@ template <int NW, int LPL, class Src>
 static cudaError_t launch_t(const Src& src, int D, int grid, const Method& mt, cudaStream_t s) {
   return launch_agg(D == 2 * NW * LPL ? planar_row_kernel<NW, LPL, true, Src>
                                       : planar_row_kernel<NW, LPL, false, Src>,
-                    grid, kPairThreads, 2 * planar_row_smem(NW), s, std::is_same<Src, OnePair>::value, src, mt);
+                    grid, kPairThreads, 2 * planar_ring_smem(D, LPL), s, std::is_same<Src, OnePair>::value, src, mt);
 }
 
 template <class Src>

@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(kPairThreads)
   const bool back = threadIdx.x >= 32;
   int item = blockIdx.x;
   const Problem pb = src.locate(item);
-  planar_long<NW, FULL>(pb, mt, item, back, shm + (back ? planar_row_smem(NW) : 0));
+  planar_long<NW, FULL>(pb, mt, item, back, shm + (back ? planar_ring_smem(pb.D, 32) : 0));
   launch_dependents();
   wait_prerequisites();
 }
@@ -52,7 +52,7 @@ static cudaError_t launch_planar_long_w(const Src& src, int D, int grid, const M
                                         cudaStream_t s) {
   return launch_agg(D == 64 * NW ? planar_long_kernel<NW, true, Src>
                                  : planar_long_kernel<NW, false, Src>,
-                    grid, kPairThreads, 2 * planar_row_smem(NW), s, true, src, mt);
+                    grid, kPairThreads, 2 * planar_ring_smem(D, 32), s, true, src, mt);
 }
 template <class Src>
 static cudaError_t launch_planar_long_t(const Src& src, int D, int grid, const Method& mt,

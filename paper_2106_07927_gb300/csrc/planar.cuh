@@ -77,11 +77,14 @@ __host__ __device__ inline int planar_planes(const Method& mt) {
 }
 
 // ------------------------------------------------------------------------------- rows
-// Costs of a row (and the other direction's U) are copied to shared memory kRowChunk pixels at a
+// Costs of a row (and the other direction's U) are copied to shared memory a chunk of pixels at a
 // time (one contiguous run), three chunks ahead.
-constexpr int kRowChunk = 8, kRowStages = 4;
-__host__ __device__ inline int planar_row_smem(int nw) {  // of one warp
-  return 2 * kRowStages * kRowChunk * 64 * nw;
+constexpr int kRowStages = 4, kRowChunk = 8;
+// Ring of one warp of 32 / lpl chains: what their D takes, since it decides how many blocks of both
+// kernels share an SM (803 x 601, D = 144: 350 -> 314 us a call against rings for full lanes; chunks of
+// 4 pixels at D > 128: 2513 x 122, D = 240 380 -> 415).
+__host__ __device__ inline int planar_ring_smem(int D, int lpl) {
+  return 2 * kRowStages * kRowChunk * (32 / lpl) * D;
 }
 // Warps of one direction: 32 / lanes rows each.
 __host__ __device__ inline int planar_row_warps(int H, int lpl) {
@@ -196,8 +199,8 @@ struct LongChain {
   }
 };
 
-// Rows y0 .. y0 + 32 / LPL - 1 in one direction, one per group of LPL lanes. ring:
-// planar_row_smem(NW) bytes of this warp. The two directions meet at pixel `mid` (a multiple of the
+// Rows y0 .. y0 + 32 / LPL - 1 in one direction, one per group of LPL lanes. ring: planar_ring_smem
+// bytes of this warp. The two directions meet at pixel `mid` (a multiple of the
 // chunk) when they share a plane.
 template <int NW, int LPL, bool FULL, bool BACK>
 __device__ __forceinline__ void planar_rows(const Problem& pb, const Method& mt, int y0,
@@ -209,6 +212,7 @@ __device__ __forceinline__ void planar_rows(const Problem& pb, const Method& mt,
   const int y = y0 + c;
   LongChain<NW, LPL, FULL> chain(lane, D);
   const bool valid = y < pb.H, active = valid && chain.owns;
+  const int at = chain.owns ? lig * 2 * NW : 0;  // the lane's bytes of a pixel (else: never used)
   const bool paired = planar_paired(mt);
   const int64_t row = (int64_t)(valid ? y : 0) * W * D;
   const uint32_t slot_bytes = (uint32_t)(CPW * G * D);
@@ -264,8 +268,8 @@ __device__ __forceinline__ void planar_rows(const Problem& pb, const Method& mt,
       __syncwarp();
       const int n = min(G, len - k * G);
       const uint32_t slot = ring_s + (uint32_t)(k & (kRowStages - 1)) * slot_bytes +
-                            (uint32_t)(lig * 2 * NW + (BACK ? (n - 1) * D : 0));
-      uint8_t* out = plane + (int64_t)(first(k, n) + (BACK ? n - 1 : 0)) * D + lig * 2 * NW;
+                            (uint32_t)(at + (BACK ? (n - 1) * D : 0));
+      uint8_t* out = plane + (int64_t)(first(k, n) + (BACK ? n - 1 : 0)) * D + at;
       if (n == G) {
         typename PB::T raw[G], oth[G];
 #pragma unroll
@@ -534,7 +538,7 @@ __device__ __forceinline__ void planar_shear(const Problem& pb, const Method& mt
 
 // One direction of sheared chain `item` (all chains of kind pair 0, then of 1 and 2), the whole warp
 // on one chain. Costs are copied kRowChunk steps at a time, three chunks ahead, each lane the same
-// 16-byte pieces of every chunk. W >= kRowChunk. ring: planar_row_smem(NW) bytes of this warp.
+// 16-byte pieces of every chunk. W >= kRowChunk. ring: planar_ring_smem bytes of this warp.
 template <int NW, bool FULL>
 __device__ __forceinline__ void planar_long(const Problem& pb, const Method& mt, int item,
                                             bool back, uint8_t* ring) {
@@ -549,6 +553,7 @@ __device__ __forceinline__ void planar_long(const Problem& pb, const Method& mt,
   const int dy = back ? -1 : 1, dx = back ? -sh : sh;
   const int ystart = back ? H - 1 : 0;
   LongChain<NW, 32, FULL> chain(lane, D);
+  const int at = chain.owns ? lane * 2 * NW : 0;  // the lane's bytes of a pixel (else: never used)
   const uint32_t P1P1 = (uint32_t)mt.P1 * 0x10001u, P2P2 = (uint32_t)mt.P2 * 0x10001u;
   const uint32_t slot_bytes = (uint32_t)(G * D);
   const uint32_t other = kRowStages * slot_bytes;  // the other direction's U behind the costs
@@ -614,7 +619,7 @@ __device__ __forceinline__ void planar_long(const Problem& pb, const Method& mt,
     auto step = [&](typename PB::T raw, typename PB::T oth, uint32_t o) {
       typename PB::T u = chain.step(raw, P1P1, P2P2);
       if (add) PB::add(u, oth);  // bytes add without a carry
-      uint8_t* const out = plane + o + lane * 2 * NW;
+      uint8_t* const out = plane + o + at;
       if (chain.owns && R2T_CHECKED(pb, out, 2 * NW, pb.agg, planar_planes(mt) * nde, 4))
         PB::store(out, u);
     };
@@ -626,7 +631,7 @@ __device__ __forceinline__ void planar_long(const Problem& pb, const Method& mt,
       asm volatile("cp.async.wait_group 3;" ::: "memory");
       __syncwarp();
       const uint32_t slot = ring_s + (uint32_t)(k & (kRowStages - 1)) * slot_bytes +
-                            (uint32_t)(lane * 2 * NW);
+                            (uint32_t)at;
       const int m = min(G, n - k * G);
       const int last = x + G * dx;
       if (m == G && !fresh && last < W && last >= 0) {  // no line starts in or after the chunk

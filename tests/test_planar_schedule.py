@@ -179,3 +179,32 @@ def test_selection_scans_every_sum_once(W, D, T):
                 kb, w = kb + 16, w + 16 * (2 * pitch + 1)
     want = {(x, d): [x - d] for x in range(W) for d in range(min(D, x + 1))}
     assert seen == want
+
+
+@pytest.mark.parametrize("D", range(16, 257, 16))
+def test_ring_accesses_stay_inside(D):
+    # shared-memory reads and copies of the row walk and of the walk with one chain per warp, in the
+    # bytes planar_ring_smem gives one warp: 2 x 4 slots of 8 pixels of each chain
+    shapes, G = [(1 if D <= 64 else 2 if D <= 128 else 4, 32)], 8  # one chain per warp
+    for dpl in (2, 4, 8):
+        if D // dpl <= 32:
+            lanes = 8
+            while lanes < D // dpl:
+                lanes *= 2
+            shapes.append((dpl // 2, lanes))
+    for nw, lpl in shapes:
+        cpw = 32 // lpl
+        size = 2 * 4 * G * cpw * D
+        slot_bytes, other = cpw * G * D, 4 * cpw * G * D
+        for lane in range(32):
+            c, lig = lane // lpl, lane % lpl
+            at = lig * 2 * nw if lig < D // (2 * nw) else 0
+            for stage in (0, 3):
+                base = c * G * D + stage * slot_bytes + other
+                assert base + (G - 1) * D + at + 2 * nw <= size
+                for v in range(nw):
+                    i = lig + lpl * v
+                    if i < G * D // 16:
+                        assert base + 16 * i + 16 <= size
+        # every piece of a chunk is copied by some lane
+        assert {lig + lpl * v for lig in range(lpl) for v in range(nw)} >= set(range(G * D // 16))
