@@ -115,8 +115,8 @@ typedef struct res2tac_pair {
  *   row_mode 2 and D = 32 agg_dpl only, other settings read the volume).
  * Automatic values: agg_dpl 2 for D <= 64, 4 for D <= 128, else 8; agg_warps 2; row_mode 2;
  * cost_mode 1 (measured faster); row_cost 1; for a context on path planes (see res2tac_create)
- * wta_chunk 64, shear_cpl 1 and shear_dpl 8 on small images, else 16; otherwise wta_chunk 128,
- * shear_dpl 16, shear_cpl 2 at D = 128, else 1.
+ * shear_cpl 1 and shear_dpl 8 on small images, else 16; otherwise shear_dpl 16, shear_cpl 2 at D =
+ * 128, else 1; wta_chunk 128 (on path planes at most what 29 KB of sums hold).
  * A context on path planes uses them for calls with shear_dpl 8 or 16, shear_cpl 1, row_mode 2,
  * cost_mode 1 and row_cost 1 (agg_warps has no effect there), and adds its sums in place with any
  * other setting. */
@@ -276,8 +276,8 @@ int res2tac_autotune(res2tac_t h, const uint8_t* left, const uint8_t* right, int
  *   shear_dpl, shear_cpl  disparities and chains per lane of the column and diagonal paths:
  *              (16, 1) or (16, 2)
  *   wta_px     pixels per WTA / right-disparity tile: 64, 128 or 256 (fewer when the tile's sums
- *              would exceed 64 KB; half as many on path planes, where shear_dpl and shear_cpl have
- *              no effect)
+ *              would exceed 64 KB, on path planes 29 KB; shear_dpl and shear_cpl have no effect
+ *              there)
  * Defaults: row_dpl 2 / 4 / 8 for D <= 64 / <= 128 / larger, (16, 1), 128. */
 typedef struct res2tac_batch_tuning {
   int32_t max_disp, large;

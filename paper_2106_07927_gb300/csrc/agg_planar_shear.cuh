@@ -7,7 +7,7 @@
 namespace r2t {
 
 template <int NL, class Src>
-__global__ void __launch_bounds__(kPairThreads)
+__global__ void __launch_bounds__(kPairThreads, 16)  // 64 registers a thread
     planar_shear_kernel(const __grid_constant__ Src src, Method mt) {
   extern __shared__ __align__(16) uint8_t shm[];
   const bool back = threadIdx.x >= 32;

@@ -636,7 +636,7 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
     }
     if (pg.p[0].planar) {
       const BatchTune& tn = tune(order[g.first]);
-      c = run_group(pg, mt, tn.row_dpl, tn.wta_px / 2, st);
+      c = run_group(pg, mt, tn.row_dpl, tn.wta_px, st);
       total += 6;
     } else {
       int l = 0;

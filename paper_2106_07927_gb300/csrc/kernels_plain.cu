@@ -135,9 +135,6 @@ Tuning default_planar_tuning(int W, int D, int num_paths) {
   Tuning t = default_tuning(D);
   t.shear_dpl = planar_shear_dpl(2 * planar_long_pairs(W, num_paths), W);
   t.shear_cpl = 1;
-  // 1242 x 375, D = 128: tiles of 64 pixels 0.051 ms, of 128 0.057 (1920 x 1080, D = 256: 0.455,
-  // 0.480)
-  t.wta_chunk = 64;
   return t;
 }
 

@@ -685,9 +685,13 @@ __device__ __forceinline__ void planar_long(const Problem& pb, const Method& mt,
 // (D^R), 16 words at a time with the word's number in the low 4 bits of each half, so one
 // instruction adds the number and takes the minimum of two sums; the least key has the least
 // sum and, among equal ones, the smallest d.
+// Pixels of a tile: whole blocks of 16 words along a diagonal, at most T and at most 29 KB of sums, past
+// which the SM has too little left for the L1, which holds the loads in flight. Stage us at 1281 x
+// 720 with 32, 64, 96, 128 pixels: D = 48 95, 64, -, 52; D = 64 98, 68, -, 59; D = 128 121, 101, 99, 115;
+// D = 160 146, 129, 152, -; D = 224 182, 166, 174, -; D = 256 195, 214, 220, -.
 __host__ __device__ inline int planar_wta_px(int D, int T) {
-  const int cap = (73728 / (2 * D)) & ~31;  // whole blocks of 16 words along a diagonal
-  return T < cap ? T : cap;                 // at most about 36 KB of sums
+  const int cap = (29500 / (4 * (D / 2 + 1))) & ~31;
+  return T < cap ? T : cap;
 }
 __host__ __device__ inline size_t planar_wta_smem(int D, int T) {
   return (size_t)T * (D / 2 + 1) * 4 + (size_t)(T + D) * 8;
