@@ -15,7 +15,7 @@
 //
 // ncc_stats_kernel: per pixel, the patch sum and the factor (iA for the reference image, jB for
 // the matching one), as one 8-byte pair, and the exact variance v.
-// ncc_cost_kernel: a band of kNccTY rows x TX pixels x all D per block of 256 threads; thread
+// ncc_cost_kernel: a band of TY rows (ncc_band) x TX pixels x all D per block of 256 threads; thread
 // (x, g) owns disparities 4g .. 4g + 3 of pixel x. Down the band it forms, per image row, the
 // dot products of the patch rows (dp4a over byte words realigned from shared memory) and keeps
 // the last n of them in a register ring, so sum a b over the patch costs one row of work per
@@ -29,12 +29,40 @@ namespace r2t {
 
 namespace {
 
-constexpr int kNccTY = 32;                        // output rows per block
-constexpr int kNccMaxRows = kNccTY + 8;           // staged rows, n <= 9
+constexpr int kNccMaxTY = 64;                     // most output rows per block
 constexpr int kNccLStride = 80;                   // >= TX + 2r + 8 for TX <= 64
 constexpr int kNccRStride = 288;                  // >= TX + D - 1 + 2r + 3 + 8 for D <= 256
 
 __host__ __device__ inline int ncc_tx(int D) { return 256 / (D / 4); }  // pixels per block
+
+// Shared memory of a block: TY + n - 1 staged rows of both images, and for 9 x 9 the ring.
+inline size_t ncc_smem(int n, int TY) {
+  return (size_t)(TY + n - 1) * (kNccLStride + kNccRStride) + (n > 5 ? (size_t)n * 256 * 16 : 0);
+}
+
+// Output rows of a block. A block computes n - 1 rows of dot products more than it outputs, so long
+// bands are cheaper, but the last wave of blocks should be full: the band with the least waves x
+// (TY + n - 1 rows + about 4 rows' worth of staging). Stage us, 9 x 9, against bands of 32 rows: 640
+// x 480, D = 64 87 -> 77; 1242 x 375, D = 128 189 -> 185; 1920 x 1080, D = 256 1347 -> 1309; 5 x 5, 350
+// x 260, D = 112 51 -> 44.
+int ncc_band(int W, int H, int D, int n) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t fit = (int64_t)std::max(sms, 1) * (n == 5 ? 4 : 3);  // blocks at a time
+  const int64_t ntx = (W + ncc_tx(D) - 1) / ncc_tx(D);
+  int best = 16;
+  int64_t least = INT64_MAX;
+  for (int TY = 16; TY <= kNccMaxTY; TY++) {
+    const int64_t waves = (ntx * ((H + TY - 1) / TY) + fit - 1) / fit;
+    const int64_t cost = waves * (std::min(TY, H) + n - 1 + 4);
+    if (cost < least) {
+      least = cost;
+      best = TY;
+    }
+  }
+  return best;
+}
 
 // Patch sum and factor of every pixel of one image (blocks of 32 x 8): {sum a, bits of f} with
 // f = 1 / sqrt(float(vA)) (reference image) or 255 / ... as fl(255 * f) (matching image, scale255).
@@ -112,17 +140,20 @@ __device__ __forceinline__ uint32_t ncc_round(float q) {
 
 template <int N_>
 __global__ void __launch_bounds__(256, N_ == 5 ? 4 : 3)
-    ncc_cost_kernel(Problem pb, int agg_bytes_per_de, const uint2* st, const int32_t* sv) {
+    ncc_cost_kernel(Problem pb, int agg_bytes_per_de, const uint2* st, const int32_t* sv, int TY) {
   constexpr int R = N_ / 2;
   constexpr int NW = (N_ + 3) / 4;  // dot-product words of a patch row
-  __shared__ __align__(16) uint8_t sl[kNccMaxRows][kNccLStride];
-  __shared__ __align__(16) uint8_t sr[kNccMaxRows][kNccRStride];
-  extern __shared__ __align__(16) uint8_t sst_ring[];  // 9 x 9: N_ x 256 x 16 bytes of ring
+  // 9 x 9: N_ x 256 x 16 bytes of ring, then the staged rows
+  extern __shared__ __align__(16) uint8_t sst_ring[];
+  uint8_t* const staged = sst_ring + (N_ > 5 ? N_ * 256 * 16 : 0);
+  uint8_t(*const sl)[kNccLStride] = reinterpret_cast<uint8_t(*)[kNccLStride]>(staged);
+  uint8_t(*const sr)[kNccRStride] =
+      reinterpret_cast<uint8_t(*)[kNccRStride]>(staged + (TY + 2 * R) * kNccLStride);
   const int W = pb.W, H = pb.H, D = pb.D;
   const int TX = ncc_tx(D), G = D / 4;
   const int ntx = (W + TX - 1) / TX;
-  const int x0 = (blockIdx.x % ntx) * TX, y0 = (blockIdx.x / ntx) * kNccTY;
-  const int nrows = min(kNccTY, H - y0) + 2 * R;  // staged rows y0 - R .. y0 + ny - 1 + R
+  const int x0 = (blockIdx.x % ntx) * TX, y0 = (blockIdx.x / ntx) * TY;
+  const int nrows = min(TY, H - y0) + 2 * R;  // staged rows y0 - R .. y0 + ny - 1 + R
   const int lbase = x0 - R;                       // image column of sl[.][0]
   const int rbase = x0 - (D - 1) - R - 3;         // image column of sr[.][0]
   const int lw = TX + 2 * R + 8, rw = TX + D - 1 + 2 * R + 3 + 8;
@@ -161,7 +192,7 @@ __global__ void __launch_bounds__(256, N_ == 5 ? 4 : 3)
   // clear the aggregated sums and reset the right-disparity keys of the tile's pixels: per row
   // one contiguous run of nx pixels (16-byte pieces, D % 16 == 0)
   {
-    const int ny = min(kNccTY, H - y0), nx = min(TX, W - x0);
+    const int ny = min(TY, H - y0), nx = min(TX, W - x0);
     const int pieces = nx * D * agg_bytes_per_de / 16;
     for (int row = 0; row < ny; row++) {
       const int64_t p = (int64_t)(y0 + row) * W + x0;
@@ -299,12 +330,12 @@ cudaError_t launch_ncc_n(const Problem& pb, const Method& mt, cudaStream_t s) {
   ncc_stats_kernel<N_><<<sg, 256, 0, s>>>(pb.right, pb.in_pitch, pb.W, pb.H, pb.nst + npx,
                                           pb.nsv + npx, true);
   const int TX = ncc_tx(pb.D);
-  const int blocks = ((pb.W + TX - 1) / TX) * ((pb.H + kNccTY - 1) / kNccTY);
-  const int ring_smem = N_ > 5 ? N_ * 256 * 16 : 0;
-  if (ring_smem)
-    cudaFuncSetAttribute(ncc_cost_kernel<N_>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         ring_smem);
-  ncc_cost_kernel<N_><<<blocks, 256, ring_smem, s>>>(pb, mt.wide ? 4 : 2, pb.nst, pb.nsv);
+  const int TY = ncc_band(pb.W, pb.H, pb.D, N_);
+  const int blocks = ((pb.W + TX - 1) / TX) * ((pb.H + TY - 1) / TY);
+  const size_t smem = ncc_smem(N_, TY);
+  cudaFuncSetAttribute(ncc_cost_kernel<N_>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)ncc_smem(N_, kNccMaxTY));
+  ncc_cost_kernel<N_><<<blocks, 256, smem, s>>>(pb, mt.wide ? 4 : 2, pb.nst, pb.nsv, TY);
   return cudaGetLastError();
 }
 
