@@ -278,7 +278,8 @@ int res2tac_autotune(res2tac_t h, const uint8_t* left, const uint8_t* right, int
  *   wta_px     pixels per WTA / right-disparity tile: 64, 128 or 256 (fewer when the tile's sums
  *              would exceed 64 KB, on path planes 29 KB; shear_dpl and shear_cpl have no effect
  *              there)
- * Defaults: row_dpl 2 / 4 / 8 for D <= 64 / <= 128 / larger, (16, 1), 128. */
+ * Defaults: row_dpl 2 / 4 / 8 for D <= 64 / <= 128 / larger (8 for D <= 64 on path planes), (16, 1),
+ * 128. */
 typedef struct res2tac_batch_tuning {
   int32_t max_disp, large;
   int32_t row_dpl, shear_dpl, shear_cpl, wta_px;

@@ -578,7 +578,7 @@ size_t res2tac_batch_workspace_bytes(const res2tac_params* p, const res2tac_pair
 
 int res2tac_batch_reserve(res2tac_t h, size_t scratch_bytes, int32_t max_pairs) {
   if (!h || max_pairs < 1) return fail(RES2TAC_EINVAL, "bad batch reservation");
-  int rc = r2t::batch_reserve(&h->batch, scratch_bytes, max_pairs);
+  int rc = r2t::batch_reserve(&h->batch, scratch_bytes, max_pairs, r2t::batch_planar_method(h->method));
   if (rc == 0) h->batch_reserved = 1;
   if (rc == -2) return fail(RES2TAC_ENOMEM, "batch reservation of %zu bytes failed", scratch_bytes);
   if (rc) return fail(RES2TAC_ECUDA, "batch reservation: %s", r2t::batch_error(h->batch));
@@ -606,7 +606,7 @@ int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res
     offs[i] = total;
     total += layout_for(q.width, q.height, q.max_disp, wide).total;
   }
-  int rc = r2t::batch_reserve(&h->batch, total, n);
+  int rc = r2t::batch_reserve(&h->batch, total, n, r2t::batch_planar_method(h->method));
   if (rc == -2) return fail(RES2TAC_ENOMEM, "batch scratch of %zu bytes could not be allocated", total);
   if (rc) return fail(RES2TAC_ECUDA, "batch engine setup failed: %s", r2t::batch_error(h->batch));
   char* base = r2t::batch_scratch(h->batch);
@@ -640,7 +640,7 @@ static int bucket_of(const res2tac_batch_tuning* t) {
 
 static int ensure_engine(res2tac_t h) {
   if (h->batch) return RES2TAC_OK;
-  int rc = r2t::batch_reserve(&h->batch, 0, 1);
+  int rc = r2t::batch_reserve(&h->batch, 0, 1, r2t::batch_planar_method(h->method));
   if (rc == -2) return fail(RES2TAC_ENOMEM, "batch engine setup: out of memory");
   if (rc) return fail(RES2TAC_ECUDA, "batch engine setup failed: %s", r2t::batch_error(h->batch));
   return RES2TAC_OK;
@@ -681,7 +681,7 @@ int res2tac_get_batch_tuning(res2tac_t h, res2tac_batch_tuning* t) {
   if (!h || !t) return fail(RES2TAC_EINVAL, "NULL argument");
   const int b = bucket_of(t);
   if (b < 0) return fail(RES2TAC_EINVAL, "bucket D %d large %d invalid", t->max_disp, t->large);
-  const r2t::BatchTune v = r2t::batch_get_tune(h->batch, b);
+  const r2t::BatchTune v = r2t::batch_get_tune(h->batch, b, r2t::batch_planar_method(h->method));
   t->row_dpl = v.row_dpl;
   t->shear_dpl = v.shear_dpl;
   t->shear_cpl = v.shear_cpl;
@@ -733,7 +733,7 @@ int res2tac_autotune_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, re
   std::sort(work.begin(), work.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
   int rc = ensure_engine(h);
   if (rc) return rc;
-  for (const auto& w : work) r2t::batch_set_tune(h->batch, w.second, r2t::batch_default_tune(w.second));
+  for (const auto& w : work) r2t::batch_set_tune(h->batch, w.second, r2t::batch_default_tune(w.second, r2t::batch_planar_method(h->method)));
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return fail(RES2TAC_ECUDA, "cudaEventCreate failed");
@@ -745,7 +745,7 @@ int res2tac_autotune_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, re
     const int b = work[wi].second;
     for (int param = 0; param < 3 && !rc; param++) {
       const int ncand = param == 1 ? 2 : 3;
-      r2t::BatchTune keep = r2t::batch_get_tune(h->batch, b);
+      r2t::BatchTune keep = r2t::batch_get_tune(h->batch, b, r2t::batch_planar_method(h->method));
       for (int c = 0; c < ncand && !rc; c++) {
         r2t::BatchTune t = keep;
         if (param == 0) t.row_dpl = (signed char)rows[c];
@@ -755,7 +755,7 @@ int res2tac_autotune_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, re
         }
         if (param == 2) t.wta_px = (short)wpx[c];
         if (memcmp(&t, &keep, sizeof(t)) == 0 || !r2t::batch_tune_valid(b, t)) continue;
-        const r2t::BatchTune prev = r2t::batch_get_tune(h->batch, b);
+        const r2t::BatchTune prev = r2t::batch_get_tune(h->batch, b, r2t::batch_planar_method(h->method));
         r2t::batch_set_tune(h->batch, b, t);
         const float ms = time_batch(h, pairs, n, st, e0, e1, &rc);
         if (!rc && ms < best) {
@@ -772,7 +772,7 @@ int res2tac_autotune_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, re
   int k = 0;
   for (size_t wi = 0; wi < work.size() && table && k < cap; wi++, k++) {
     const int b = work[wi].second;
-    const r2t::BatchTune v = r2t::batch_get_tune(h->batch, b);
+    const r2t::BatchTune v = r2t::batch_get_tune(h->batch, b, r2t::batch_planar_method(h->method));
     table[k].max_disp = 16 * (b / 2);
     table[k].large = b & 1;
     table[k].row_dpl = v.row_dpl;

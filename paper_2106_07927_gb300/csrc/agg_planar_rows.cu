@@ -26,7 +26,8 @@ template <int NW, int LPL, class Src>
 static cudaError_t launch_t(const Src& src, int D, int grid, const Method& mt, cudaStream_t s) {
   return launch_agg(D == 2 * NW * LPL ? planar_row_kernel<NW, LPL, true, Src>
                                       : planar_row_kernel<NW, LPL, false, Src>,
-                    grid, kPairThreads, 2 * planar_ring_smem(D, LPL), s, std::is_same<Src, OnePair>::value, src, mt);
+                    grid, kPairThreads, 2 * planar_ring_smem(D, LPL), s,
+                    std::is_same<Src, OnePair>::value, src, mt);
 }
 
 template <class Src>

@@ -13,9 +13,10 @@ struct BatchEngine;
 // Device bytes of the descriptor tables for n pairs (upper bound, excluding per-pair scratch).
 size_t batch_fixed_bytes(int n);
 
-// Creates or grows the engine so it holds scratch_bytes of per-pair scratch and n pairs.
+// Creates or grows the engine so it holds scratch_bytes of per-pair scratch and n pairs. planar: the
+// method's route (batch_planar_method), for the default settings.
 // Returns 0, -2 when device memory is short, -3 on another CUDA error.
-int batch_reserve(BatchEngine** e, size_t scratch_bytes, int n);
+int batch_reserve(BatchEngine** e, size_t scratch_bytes, int n, bool planar);
 
 // Base of the per-pair scratch (valid after batch_reserve).
 char* batch_scratch(BatchEngine* e);
@@ -35,10 +36,10 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
 
 // Kernel settings per bucket of pairs (tune_bucket: D / 16 and the size class): the defaults,
 // their validity, and the engine's table (set returns -1 for an invalid setting).
-BatchTune batch_default_tune(int bucket);
+BatchTune batch_default_tune(int bucket, bool planar);
 bool batch_tune_valid(int bucket, const BatchTune& t);
 int batch_set_tune(BatchEngine* e, int bucket, const BatchTune& t);
-BatchTune batch_get_tune(BatchEngine* e, int bucket);
+BatchTune batch_get_tune(BatchEngine* e, int bucket, bool planar);
 
 const char* batch_error(BatchEngine* e);
 void batch_destroy(BatchEngine* e);

@@ -177,10 +177,10 @@ static int grow_desc(BatchEngine* e, int n) {
   return 0;
 }
 
-int batch_reserve(BatchEngine** pe, size_t scratch_bytes, int n) {
+int batch_reserve(BatchEngine** pe, size_t scratch_bytes, int n, bool planar) {
   if (!*pe) {
     BatchEngine* e = new BatchEngine();
-    for (int b = 0; b < kTuneBuckets; b++) e->tune[b] = batch_default_tune(b);
+    for (int b = 0; b < kTuneBuckets; b++) e->tune[b] = batch_default_tune(b, planar);
     e->err[0] = 0;
     memset(&e->graph_method, 0, sizeof(Method));
     *pe = e;
@@ -217,11 +217,15 @@ int batch_reserve(BatchEngine** pe, size_t scratch_bytes, int n) {
 char* batch_scratch(BatchEngine* e) { return e ? e->scratch : nullptr; }
 const char* batch_error(BatchEngine* e) { return e ? e->err : "no batch engine"; }
 
-BatchTune batch_default_tune(int bucket) {
+BatchTune batch_default_tune(int bucket, bool planar) {
   const int D = 16 * (bucket / 2);
   BatchTune t;
   memset(&t, 0, sizeof(t));
-  t.row_dpl = (signed char)long_dpl_default(D);
+  // On path planes a group has warps enough to hide the row steps' latency, so at D <= 64 the shape
+  // with the fewest instructions: 64 x 320x240, D = 64 1357 us with 2 disparities per lane, 1324 with 8
+  // (small batches: see batch_run_planar). At larger D the single pair's: of seven uneven batches
+  // 8 at D = 128 was up to 2 % slower on three and up to 1.2 % faster on four.
+  t.row_dpl = (signed char)(planar && D <= 64 ? 8 : long_dpl_default(D));
   t.shear_dpl = 16;
   t.shear_cpl = 1;
   t.wta_px = 128;
@@ -243,8 +247,9 @@ int batch_set_tune(BatchEngine* e, int bucket, const BatchTune& t) {
   return 0;
 }
 
-BatchTune batch_get_tune(BatchEngine* e, int bucket) {
-  return (e && bucket >= 0 && bucket < kTuneBuckets) ? e->tune[bucket] : batch_default_tune(bucket);
+BatchTune batch_get_tune(BatchEngine* e, int bucket, bool planar) {
+  return (e && bucket >= 0 && bucket < kTuneBuckets) ? e->tune[bucket]
+                                                     : batch_default_tune(bucket, planar);
 }
 
 void batch_destroy(BatchEngine* e) {
@@ -613,6 +618,11 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
     for (int k = 0; k < slots && c == cudaSuccess; k++)
       c = cudaStreamWaitEvent(e->main[k], e->ev_start, 0);
   }
+  // a batch with few rows leaves the row steps' latency open: at most the single pair's setting
+  // (2 x 640x480, D = 64: 254 us with 2 disparities per lane, 260 with 8)
+  int64_t rows = 0;
+  for (int i = 0; i < n; i++) rows += probs[i].H;
+  const bool few = rows <= 1250;
   int total = 0;
   PairGroup pg;
   for (int gi = 0; gi < G && c == cudaSuccess; gi++) {
@@ -636,7 +646,8 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
     }
     if (pg.p[0].planar) {
       const BatchTune& tn = tune(order[g.first]);
-      c = run_group(pg, mt, tn.row_dpl, tn.wta_px, st);
+      const int dpl = few ? std::min((int)tn.row_dpl, long_dpl_default(pg.p[0].D)) : tn.row_dpl;
+      c = run_group(pg, mt, dpl, tn.wta_px, st);
       total += 6;
     } else {
       int l = 0;
