@@ -8,8 +8,8 @@ same JSON line:
   - e2e: four pairs of the workload in turn through res2tac_compute_host from pinned host
     buffers (transfers, compute, synchronise; L2 flushed before each step), as the paper times
     its pipeline, and the same with one staged cudaMemcpyAsync per image and for the map;
-  - batched: 64 pairs of uneven W, H, D in one res2tac_compute_batch call (persistent kernels
-    under a CUDA graph) vs the same 64 pairs as per-pair res2tac_compute launches;
+  - batched: 64 pairs of uneven W, H, D in one res2tac_compute_batch call (one launch per stage
+    and group of pairs) vs the same 64 pairs as per-pair res2tac_compute launches;
   - serving: 10,000 Poisson arrivals (the batch sizes plus 5 % 3840x2160, D = 256) at each of
     200, 500, 1000, 2000 and 5000 pairs/s through the continuous-batching server, p50 / p99 /
     p99.9 latency per rate; a 1 % sample checked against the CPU oracle after the sweep;
@@ -660,14 +660,15 @@ def main():
                                  if args.pair is None else None),
                      "ops_per_launch": ops_agg, "algorithmic_bytes_per_launch": bytes_agg,
                      "dominant_stage": dominant,
-                     # the accumulation into S: every path adds 2 bytes per DE (read-modify-write
-                     # in L2), against the measured rate of bulk add-reductions
-                     "s_accumulation": {
-                         "bytes_per_launch": 2 * de * prm["num_paths"],
-                         "achieved_gbs": round(2 * de * prm["num_paths"] / (agg_ms / 1e3) / 1e9, 1),
-                         "peak_gbs": round(red_peak / 1e9, 1),
-                         "frac": round(2 * de * prm["num_paths"] / (agg_ms / 1e3) / red_peak, 3),
-                         "peak_source": "measured TMA bulk add-reduction probe, S-sized buffer"}},
+                     # bytes between the SMs and the L2: every path reads the cost (1 B per DE) and
+                     # stores its term (1 B), and half of the terms of each pair of opposite
+                     # paths' shared plane are read back and stored again as sums (2 P2 <= 255)
+                     "l2_bytes": {
+                         "bytes_per_launch": de * prm["num_paths"] * 5 // 2,
+                         "achieved_gbs": round(de * prm["num_paths"] * 2.5 / (agg_ms / 1e3) / 1e9,
+                                               1),
+                         "red_probe_gbs": round(red_peak / 1e9, 1),
+                         "red_probe": "measured TMA bulk add-reduction probe, for comparison"}},
         # recomputing the cost inside each path walk instead of reading the volume: two 32-bit
         # POPC per DE and path at the measured POPC rate, against the aggregation's own time
         "cost_recompute_bound": {
