@@ -224,11 +224,14 @@ int res2tac_compute_raw(res2tac_t h, const uint8_t* raw_left, const uint8_t* raw
  * its sums in place. Otherwise the groups hold at most 96 MB of cost and aggregated volumes, run
  * as persistent kernels fed by device work queues and the whole batch is one CUDA graph, captured
  * once per group count and replayed while the capacities last.
- * res2tac_last_launch_count: 6 per group. The context grows its batch scratch when a larger batch
- * arrives (unless res2tac_batch_reserve sized it, to more than res2tac_batch_workspace_bytes only
- * for a pair's planes and where half of the device's memory stays free): that call allocates and
- * must not be made during stream capture. No block of either route ever waits for another one of
- * another launch, so there is no device-side wait that could time out: RES2TAC_ETIMEOUT is reserved
+ * res2tac_last_launch_count: 6 per group. The context allocates its batch scratch anew only when
+ * a larger batch arrives (by res2tac_batch_workspace_bytes), then with room for the planes of the
+ * batch's largest pair where half of the device's memory stays free (not after
+ * res2tac_batch_reserve): that call allocates and must not be made during stream capture. A call
+ * captured into a graph can be replayed until such a batch arrives; with p2 <= 255 the graph holds
+ * the batch's descriptors. The blocks of a launch wait only for kernels launched before it, never
+ * for work that is yet to come, so there is no device-side wait that could time out:
+ * RES2TAC_ETIMEOUT is reserved
  * and not returned. RES2TAC_EINVAL for an invalid pair, or for RES2TAC_EXACT_CC / RES2TAC_NCC
  * contexts (single pairs only). */
 int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res2tac_stream_t s);

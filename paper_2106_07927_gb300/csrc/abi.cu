@@ -578,7 +578,8 @@ size_t res2tac_batch_workspace_bytes(const res2tac_params* p, const res2tac_pair
 
 int res2tac_batch_reserve(res2tac_t h, size_t scratch_bytes, int32_t max_pairs) {
   if (!h || max_pairs < 1) return fail(RES2TAC_EINVAL, "bad batch reservation");
-  int rc = r2t::batch_reserve(&h->batch, scratch_bytes, max_pairs, r2t::batch_planar_method(h->method));
+  int rc = r2t::batch_reserve(&h->batch, scratch_bytes, scratch_bytes, max_pairs,
+                              r2t::batch_planar_method(h->method));
   if (rc == 0) h->batch_reserved = 1;
   if (rc == -2) return fail(RES2TAC_ENOMEM, "batch reservation of %zu bytes failed", scratch_bytes);
   if (rc) return fail(RES2TAC_ECUDA, "batch reservation: %s", r2t::batch_error(h->batch));
@@ -593,8 +594,8 @@ int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res
                 "the exact consistency check and the NCC cost run per pair (res2tac_compute)");
   std::vector<r2t::Problem> probs((size_t)n);
   std::vector<size_t> offs((size_t)n);
-  size_t total = 0;
-  const bool wide = h->method.wide != 0;
+  size_t total = 0, want = 0;
+  const bool wide = h->method.wide != 0, planar = r2t::batch_planar_method(h->method);
   for (int i = 0; i < n; i++) {
     const res2tac_pair& q = pairs[i];
     if (!shape_ok(q.width, q.height, q.max_disp))
@@ -605,8 +606,11 @@ int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res
       return fail(RES2TAC_EINVAL, "pair %d: bad pitch", i);
     offs[i] = total;
     total += layout_for(q.width, q.height, q.max_disp, wide).total;
+    if (planar && !h->batch_reserved)  // grown on demand: room for the planes of a lone pair
+      want = std::max(want,
+                      r2t::layout_single(q.width, q.height, q.max_disp, h->method).total);
   }
-  int rc = r2t::batch_reserve(&h->batch, total, n, r2t::batch_planar_method(h->method));
+  int rc = r2t::batch_reserve(&h->batch, total, want, n, planar);
   if (rc == -2) return fail(RES2TAC_ENOMEM, "batch scratch of %zu bytes could not be allocated", total);
   if (rc) return fail(RES2TAC_ECUDA, "batch engine setup failed: %s", r2t::batch_error(h->batch));
   char* base = r2t::batch_scratch(h->batch);
@@ -622,9 +626,8 @@ int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res
     probs[i] = pb;
   }
   int launches = 0;
-  if (r2t::batch_planar_method(h->method))
-    rc = r2t::batch_run_planar(h->batch, probs.data(), n, h->method, (cudaStream_t)s,
-                               !h->batch_reserved, &launches);
+  if (planar)
+    rc = r2t::batch_run_planar(h->batch, probs.data(), n, h->method, (cudaStream_t)s, &launches);
   else
     rc = r2t::batch_run(h->batch, probs.data(), n, h->method, (cudaStream_t)s, &launches);
   h->last_launches = launches;
@@ -640,7 +643,7 @@ static int bucket_of(const res2tac_batch_tuning* t) {
 
 static int ensure_engine(res2tac_t h) {
   if (h->batch) return RES2TAC_OK;
-  int rc = r2t::batch_reserve(&h->batch, 0, 1, r2t::batch_planar_method(h->method));
+  int rc = r2t::batch_reserve(&h->batch, 0, 0, 1, r2t::batch_planar_method(h->method));
   if (rc == -2) return fail(RES2TAC_ENOMEM, "batch engine setup: out of memory");
   if (rc) return fail(RES2TAC_ECUDA, "batch engine setup failed: %s", r2t::batch_error(h->batch));
   return RES2TAC_OK;

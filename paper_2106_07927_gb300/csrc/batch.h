@@ -13,10 +13,13 @@ struct BatchEngine;
 // Device bytes of the descriptor tables for n pairs (upper bound, excluding per-pair scratch).
 size_t batch_fixed_bytes(int n);
 
-// Creates or grows the engine so it holds scratch_bytes of per-pair scratch and n pairs. planar: the
-// method's route (batch_planar_method), for the default settings.
+// Creates or grows the engine so it holds `need` bytes of per-pair scratch and n pairs. The scratch is
+// allocated anew only when it is smaller than need, and then takes `want` bytes (what path planes can
+// use) where half of the device's memory stays free with them: a batch that ran once never moves
+// it again, whatever memory has become free since, so captured batches keep their addresses until a
+// larger batch arrives. planar: the method's route (batch_planar_method), for the default settings.
 // Returns 0, -2 when device memory is short, -3 on another CUDA error.
-int batch_reserve(BatchEngine** e, size_t scratch_bytes, int n, bool planar);
+int batch_reserve(BatchEngine** e, size_t need, size_t want, int n, bool planar);
 
 // Base of the per-pair scratch (valid after batch_reserve).
 char* batch_scratch(BatchEngine* e);
@@ -28,11 +31,11 @@ int batch_run(BatchEngine* e, const Problem* probs, int n, const Method& mt, cud
 
 // The route of batches whose method has path planes (batch_planar_method): groups of pairs of one D
 // run stage by stage on up to 4 streams, each stream's groups in one part of the scratch after
-// another. Uses the engine's scratch as it is (grown first to what a lone pair takes when
-// `grow`); a pair whose planes do not fit it runs with its sums in place. Returns 0 or -3.
+// another. Uses the engine's scratch as it is; a pair whose planes do not fit it runs with its sums
+// in place. Returns 0 or -3.
 bool batch_planar_method(const Method& mt);
 int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& mt, cudaStream_t s,
-                     bool grow, int* launches);
+                     int* launches);
 
 // Kernel settings per bucket of pairs (tune_bucket: D / 16 and the size class): the defaults,
 // their validity, and the engine's table (set returns -1 for an invalid setting).

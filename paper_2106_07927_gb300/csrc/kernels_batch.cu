@@ -177,7 +177,7 @@ static int grow_desc(BatchEngine* e, int n) {
   return 0;
 }
 
-int batch_reserve(BatchEngine** pe, size_t scratch_bytes, int n, bool planar) {
+int batch_reserve(BatchEngine** pe, size_t need, size_t want, int n, bool planar) {
   if (!*pe) {
     BatchEngine* e = new BatchEngine();
     for (int b = 0; b < kTuneBuckets; b++) e->tune[b] = batch_default_tune(b, planar);
@@ -201,15 +201,23 @@ int batch_reserve(BatchEngine** pe, size_t scratch_bytes, int n, bool planar) {
   BatchEngine* e = *pe;
   if (!e->main[0] || !e->copied)
     return set_err(e, cudaErrorInitializationError, "batch engine setup");
-  if (scratch_bytes > e->scratch_cap) {
+  if (need > e->scratch_cap) {
     // the previous batch may still run on its stream: wait before freeing its scratch
     cudaDeviceSynchronize();
     cudaFree(e->scratch);
     e->scratch = nullptr;
     e->scratch_cap = 0;
-    cudaError_t c = cudaMalloc(&e->scratch, scratch_bytes);
+    size_t bytes = std::max(need, want), free_b = 0, total_b = 0;
+    if (bytes > need && (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
+                         bytes + total_b / 2 > free_b))
+      bytes = need;
+    cudaError_t c = cudaMalloc(&e->scratch, bytes);
+    if (c != cudaSuccess && bytes > need) {
+      cudaGetLastError();
+      c = cudaMalloc(&e->scratch, bytes = need);
+    }
     if (c != cudaSuccess) return set_err(e, c, "batch scratch allocation");
-    e->scratch_cap = scratch_bytes;
+    e->scratch_cap = bytes;
   }
   return grow_desc(e, n);
 }
@@ -540,7 +548,7 @@ constexpr size_t kPlanarGroupBytes = (size_t)96 << 20;
 bool batch_planar_method(const Method& mt) { return mt.P2 <= 255 && !(mt.flags & (4 | 8)); }
 
 int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& mt, cudaStream_t s,
-                     bool grow, int* launches) {
+                     int* launches) {
   auto sums = [&](int i) {
     return layout_for(probs[i].W, probs[i].H, probs[i].D, mt.wide != 0);
   };
@@ -548,27 +556,10 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
     return layout_single(probs[i].W, probs[i].H, probs[i].D, mt);
   };
   std::vector<Layout> lay((size_t)n);
-  size_t largest = 0;
   for (int i = 0; i < n; i++) {
     lay[i] = planes(i);
-    largest = std::max(largest, lay[i].total);
-  }
-  if (grow && largest > e->scratch_cap) {  // half of the device's memory stays free with it
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
-        largest + total_b / 2 <= free_b + e->scratch_cap) {
-      cudaDeviceSynchronize();  // a batch may still run in the old scratch
-      void* p = nullptr;
-      if (cudaMalloc(&p, largest) == cudaSuccess) {
-        cudaFree(e->scratch);
-        e->scratch = static_cast<char*>(p);
-        e->scratch_cap = largest;
-      }
-    }
-    cudaGetLastError();
-  }
-  for (int i = 0; i < n; i++)
     if (lay[i].total > e->scratch_cap) lay[i] = sums(i);
+  }
   // groups: pairs of one D and one setting, largest first
   std::vector<int> order((size_t)n);
   std::iota(order.begin(), order.end(), 0);
