@@ -217,23 +217,23 @@ int res2tac_compute_raw(res2tac_t h, const uint8_t* raw_left, const uint8_t* raw
 /* Runs n independent pairs of uneven sizes as one batch on stream s (the paper processes one
  * pair at a time, Sec. 2.2; batching is this library's addition). Results are bit-identical to
  * res2tac_compute on each pair alone. pairs: host array of n descriptors with device pointers.
- * With p2 <= 255 the pairs are cut into groups of one max_disp of at most 96 MB of scratch (a larger
- * pair is a group of its own); a group runs its six stages with one launch each on path planes
- * (see res2tac_create), and groups rotate over up to four streams, each with its own part of the
- * batch scratch, as many as the scratch holds. A pair whose planes do not fit the scratch runs with
- * its sums in place. Otherwise the groups hold at most 96 MB of cost and aggregated volumes, run
- * as persistent kernels fed by device work queues and the whole batch is one CUDA graph, captured
- * once per group count and replayed while the capacities last.
- * res2tac_last_launch_count: 6 per group. The context allocates its batch scratch anew only when
- * a larger batch arrives (by res2tac_batch_workspace_bytes), then with room for the planes of the
- * batch's largest pair where half of the device's memory stays free (not after
- * res2tac_batch_reserve): that call allocates and must not be made during stream capture. A call
- * captured into a graph can be replayed until such a batch arrives; with p2 <= 255 the graph holds
- * the batch's descriptors. The blocks of a launch wait only for kernels launched before it, never
- * for work that is yet to come, so there is no device-side wait that could time out:
- * RES2TAC_ETIMEOUT is reserved
- * and not returned. RES2TAC_EINVAL for an invalid pair, or for RES2TAC_EXACT_CC / RES2TAC_NCC
- * contexts (single pairs only). */
+ * With p2 <= 255 the pairs are cut into groups of one max_disp, of a quarter of the batch's estimates
+ * within 20 to 40 million (a larger pair is a group of its own); a group runs its six stages with
+ * one launch each on path planes (see res2tac_create), and groups rotate over up to four streams,
+ * each with its own part of the batch scratch, as many as the scratch holds. A pair whose planes do
+ * not fit the scratch runs with its sums in place. Otherwise the groups hold at most 96 MB of cost
+ * and aggregated volumes, run as persistent kernels fed by device work queues and the whole batch
+ * is one CUDA graph, captured once per group count and replayed while the capacities last.
+ * res2tac_last_launch_count: 6 per group. The context allocates its batch scratch anew only when a
+ * larger batch arrives (by res2tac_batch_workspace_bytes), then with at most 256 MB more for path
+ * planes, and room for the planes of the batch's largest pair (that not after
+ * res2tac_batch_reserve), where half of the device's memory stays free with it: that call allocates
+ * and must not be made during stream capture. A call captured into a graph can be replayed until
+ * such a batch arrives; with p2 <= 255 the graph holds the batch's descriptors. The blocks of a
+ * launch wait only for kernels launched before it, never for work that is yet to come, so there is
+ * no device-side wait that could time out: RES2TAC_ETIMEOUT is reserved and not returned.
+ * RES2TAC_EINVAL for an invalid pair, or for RES2TAC_EXACT_CC / RES2TAC_NCC contexts (single pairs
+ * only). */
 int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res2tac_stream_t s);
 
 /* Copies the intermediates of the last res2tac_compute on this context into caller buffers
@@ -250,14 +250,16 @@ int res2tac_debug_outputs(res2tac_t h, uint8_t* cost, uint16_t* agg, uint16_t* d
  * res2tac_create). */
 size_t res2tac_workspace_bytes(const res2tac_params* p);
 
-/* Device bytes a batch of n pairs needs on top of the context (0 if a pair is invalid). */
+/* Device bytes a batch of n pairs needs on top of the context (0 if a pair is invalid); see
+ * res2tac_compute_batch for what the scratch takes beyond it where memory is free. */
 size_t res2tac_batch_workspace_bytes(const res2tac_params* p, const res2tac_pair* pairs,
                                      int32_t n);
 
 /* Pre-allocates the context's batch engine for batches of at most max_pairs pairs whose
  * res2tac_batch_workspace_bytes is at most scratch_bytes, so that such batches allocate nothing
- * (a serving loop reserves once, then admits work by its own memory accounting). Grow-only;
- * synchronises the device when it grows. RES2TAC_ENOMEM if the memory is not available. */
+ * (a serving loop reserves once, then admits work by its own memory accounting). With p2 <= 255 it
+ * takes up to 256 MB more for path planes where half of the device's memory stays free with them.
+ * Grow-only; synchronises the device when it grows. RES2TAC_ENOMEM if the memory is not available. */
 int res2tac_batch_reserve(res2tac_t h, size_t scratch_bytes, int32_t max_pairs);
 
 /* Reads / sets the kernel configuration (RES2TAC_EINVAL for a setting the context's D cannot

@@ -576,9 +576,18 @@ size_t res2tac_batch_workspace_bytes(const res2tac_params* p, const res2tac_pair
   return total + r2t::batch_fixed_bytes(n);
 }
 
+// What the batch scratch takes on top of `total` bytes of sums so that small batches run on path
+// planes at once instead of a few pairs at a time: the planes of everything that fits `total` (2
+// to 8 bytes per estimate against the sums' 2, of 3 with the cost), at most kBatchExtra.
+static size_t batch_extra(res2tac_t h, size_t total) {
+  const int planes = r2t::method_planes(h->method);
+  return planes > 2 ? std::min(r2t::kBatchExtra, total / 3 * (planes - 2) + 65536) : 0;
+}
+
 int res2tac_batch_reserve(res2tac_t h, size_t scratch_bytes, int32_t max_pairs) {
   if (!h || max_pairs < 1) return fail(RES2TAC_EINVAL, "bad batch reservation");
-  int rc = r2t::batch_reserve(&h->batch, scratch_bytes, scratch_bytes, max_pairs,
+  int rc = r2t::batch_reserve(&h->batch, scratch_bytes,
+                              scratch_bytes + batch_extra(h, scratch_bytes), max_pairs,
                               r2t::batch_planar_method(h->method));
   if (rc == 0) h->batch_reserved = 1;
   if (rc == -2) return fail(RES2TAC_ENOMEM, "batch reservation of %zu bytes failed", scratch_bytes);
@@ -607,9 +616,10 @@ int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res
     offs[i] = total;
     total += layout_for(q.width, q.height, q.max_disp, wide).total;
     if (planar && !h->batch_reserved)  // grown on demand: room for the planes of a lone pair
-      want = std::max(want,
-                      r2t::layout_single(q.width, q.height, q.max_disp, h->method).total);
+      want = std::max(want, r2t::layout_single(q.width, q.height, q.max_disp, h->method,
+                                               r2t::kPlanarBytes, false).total);
   }
+  want = std::max(want, total + batch_extra(h, total));
   int rc = r2t::batch_reserve(&h->batch, total, want, n, planar);
   if (rc == -2) return fail(RES2TAC_ENOMEM, "batch scratch of %zu bytes could not be allocated", total);
   if (rc) return fail(RES2TAC_ECUDA, "batch engine setup failed: %s", r2t::batch_error(h->batch));

@@ -8,6 +8,13 @@
 
 namespace r2t {
 
+// Most bytes the batch scratch takes beyond the sums' layout for path planes: with none, a batch whose
+// planes do not fit runs a few pairs at a time, and small pairs then wait for one another's chains
+// (5 x 160x120, D = 32, P2 = 200: 193 us, 53 with room for all; the persistent kernels 97). Small
+// batches fit; larger ones fill the GPU a few pairs at a time (with 512 MB: 8 x 640x480, D = 32, P2 =
+// 200 571 -> 425 us, 8 x 320x240, D = 128 367 -> 335, the others within 5 %).
+constexpr size_t kBatchExtra = (size_t)256 << 20;
+
 struct BatchEngine;
 
 // Device bytes of the descriptor tables for n pairs (upper bound, excluding per-pair scratch).

@@ -540,10 +540,13 @@ int batch_run(BatchEngine* e, const Problem* probs, int n, const Method& mt, cud
 // descriptors in memory and no work queues. Against the persistent kernels above, which add into
 // 16-bit sums: 64 x 320x240, D = 64 1.78 -> 1.34 ms; 16 x 1242x375, D = 128 4.82 -> 3.83 ms; 16
 // uneven pairs up to 1920x1080, D = 256 11.9 -> 7.3 ms.
-// Scratch of one group (a larger pair is a group of its own): 64 x 320x240 took 1.80, 1.34, 1.36 and
-// 1.41 ms with 48, 96, 192 and 400 MB - larger groups fill the GPU, smaller ones stay in the L2;
-// batches of larger pairs do not depend on it.
-constexpr size_t kPlanarGroupBytes = (size_t)96 << 20;
+// Estimates (W H D) of one group: a quarter of the batch's, so that every stream has work, within these
+// bounds (a larger pair is a group of its own). Smaller groups leave the GPU to launches and to the
+// latency of the chains, larger ones the streams without work. us with groups of at least 5, 12 and
+// 20 million: 6 x 320x240, D = 64 223, 136, 137; 5 x 413x307, D = 48 233, 234, 181; 2 x 640x480, D =
+// 32 240, 240, 148. With at most 20, 40 and 60 million: 48 x 320x240, D = 128, 4 paths 1290, 1184,
+// 1191; 16 x 640x480, D = 64, 4 paths 1106, 945, 960; 64 x 320x240, D = 64 1274, 1304, 1322.
+constexpr int64_t kGroupLeast = 20000000, kGroupMost = 40000000;
 
 bool batch_planar_method(const Method& mt) { return mt.P2 <= 255 && !(mt.flags & (4 | 8)); }
 
@@ -553,7 +556,7 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
     return layout_for(probs[i].W, probs[i].H, probs[i].D, mt.wide != 0);
   };
   auto planes = [&](int i) {
-    return layout_single(probs[i].W, probs[i].H, probs[i].D, mt);
+    return layout_single(probs[i].W, probs[i].H, probs[i].D, mt, kPlanarBytes, false);
   };
   std::vector<Layout> lay((size_t)n);
   for (int i = 0; i < n; i++) {
@@ -579,13 +582,20 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
     size_t bytes;
   };
   std::vector<Group> groups;
-  const size_t most = std::min(kPlanarGroupBytes, e->scratch_cap);
+  auto estimates = [&](int i) { return (int64_t)probs[i].W * probs[i].H * probs[i].D; };
+  int64_t most = 0;
+  for (int i = 0; i < n; i++) most += estimates(i);
+  most = std::min(kGroupMost, std::max(kGroupLeast, most / kSlots));
   for (int i = 0; i < n;) {
     Group g{i, 1, lay[order[i]].total};
+    int64_t de = estimates(order[i]);
     for (i++; i < n && g.n < kGroupPairs && alike(order[g.first], order[i]) &&
-              g.bytes + lay[order[i]].total <= most;
-         i++, g.n++)
+              de + estimates(order[i]) <= most &&
+              g.bytes + lay[order[i]].total <= e->scratch_cap;
+         i++, g.n++) {
       g.bytes += lay[order[i]].total;
+      de += estimates(order[i]);
+    }
     groups.push_back(g);
   }
   std::stable_sort(groups.begin(), groups.end(),
@@ -596,6 +606,10 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
   size_t need = groups[0].bytes;
   while (slots < kSlots && slots < G && need + groups[slots].bytes <= e->scratch_cap)
     need += groups[slots++].bytes;
+  // no more of them than that number of turns needs, or the last turn leaves the GPU nearly empty
+  // (five groups, 5 x 640x480, D = 64: 474 us on 4 streams, 442 on 3)
+  const int turns = (G + slots - 1) / slots;
+  slots = (G + turns - 1) / turns;
   size_t base[kSlots] = {};
   for (int k = 1; k < slots; k++) base[k] = base[k - 1] + groups[k - 1].bytes;
   // a batch of this engine on another stream may still use the scratch (a capturing stream cannot

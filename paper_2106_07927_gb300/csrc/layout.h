@@ -25,9 +25,10 @@ constexpr size_t kPlanarBytes = (size_t)32 << 30;
 // 25 B per pixel. The exact
 // consistency check adds the swapped, flipped pair (2 B/px) and its D^L (2 B/px); the NCC cost
 // the patch statistics of both images (16 B/px) and their exact patch variances (8 B/px). With
-// planes > 0 the aggregated volume is that many byte planes, and the sub-pixel D^L takes 4 B/px.
+// planes > 0 the aggregated volume is that many byte planes, and with sub the sub-pixel D^L takes 4
+// B/px.
 inline Layout layout_for(int W, int H, int D, bool wide, bool exact = false, bool ncc = false,
-                         int planes = 0) {
+                         int planes = 0, bool sub = false) {
   const size_t npx = (size_t)W * H, nde = npx * D;
   Layout l;
   size_t o = 0;
@@ -46,7 +47,7 @@ inline Layout layout_for(int W, int H, int D, bool wide, bool exact = false, boo
     l.dp = o; o = align256(o + npx * 2);
   }
   l.dlf = 0;
-  if (planes) { l.dlf = o; o = align256(o + npx * 4); }
+  if (sub) { l.dlf = o; o = align256(o + npx * 4); }
   l.nst = l.nsv = 0;
   if (ncc) {  // 2 KB of slack in front (reads at a matching pixel x - d < 0 stay inside)
     l.nst = o + 2048; o = align256(o + 2048 + npx * 16);
@@ -56,13 +57,20 @@ inline Layout layout_for(int W, int H, int D, bool wide, bool exact = false, boo
   return l;
 }
 
-// The layout of a pair processed alone: path planes where the method's U fits a byte (census cost,
-// P2 <= 255) and the scratch stays within limit, else one volume of sums.
-inline Layout layout_single(int W, int H, int D, const Method& m, size_t limit = kPlanarBytes) {
+// Path planes of a method whose U fits a byte (census cost, P2 <= 255), else 0.
+inline int method_planes(const Method& m) {
+  if (m.P2 > 255 || (m.flags & 8)) return 0;
+  return 2 * m.P2 <= 255 ? m.num_paths / 2 : m.num_paths;
+}
+
+// The layout of a pair processed alone: path planes where the method has them and the scratch stays
+// within limit, else one volume of sums. sub: with the sub-pixel D^L (batches have none).
+inline Layout layout_single(int W, int H, int D, const Method& m, size_t limit = kPlanarBytes,
+                            bool sub = true) {
   const bool exact = (m.flags & 4) != 0, ncc = (m.flags & 8) != 0;
-  if (m.P2 <= 255 && !ncc && (size_t)W * H * D < ((size_t)1 << 32) - 65536) {
-    const Layout l =
-        layout_for(W, H, D, false, exact, false, 2 * m.P2 <= 255 ? m.num_paths / 2 : m.num_paths);
+  const int planes = method_planes(m);
+  if (planes && (size_t)W * H * D < ((size_t)1 << 32) - 65536) {
+    const Layout l = layout_for(W, H, D, false, exact, false, planes, sub);
     if (l.total <= limit) return l;
   }
   return layout_for(W, H, D, m.wide != 0, exact, ncc);

@@ -78,3 +78,31 @@ def test_batch_groups_and_scratch_limits(p2):
         for o, w in list(zip(outs, want))[-len(batch):]:
             assert np.array_equal(binding.u16(o), w)
         ctx.close()
+
+
+# pairs that a scratch of the size callers reserve holds at once: one launch per stage and group
+@pytest.mark.parametrize("n,W,H,D,p2,paths,groups", [
+    (5, 160, 120, 32, 200, 8, 1), (3, 160, 120, 32, 100, 8, 1), (2, 160, 120, 32, 100, 4, 1),
+    (8, 320, 240, 128, 200, 8, 4), (5, 640, 480, 64, 100, 8, 5), (33, 40, 24, 16, 120, 8, 2)])
+def test_reserved_small_batches_run_at_once(n, W, H, D, p2, paths, groups):
+    import torch
+    prm = scenes.params(64, 64, 64, 9, 7, 10, p2, paths, 3)
+    keep, pairs, outs = [], [], []
+    for i in range(n):
+        L, R = (torch.from_numpy(a).cuda() for a in _pair(i % 4, W, H, D))
+        o = torch.full((H, W), -1, dtype=torch.int16, device="cuda")
+        keep.append((L, R))
+        outs.append(o)
+        pairs.append(binding.res2tac_pair(L.data_ptr(), R.data_ptr(), W, o.data_ptr(), 2 * W, W, H,
+                                          D, 0))
+    ctx = binding.Stereo(prm)
+    binding.res2tac_batch_reserve(ctx.handle, binding.res2tac_batch_workspace_bytes(
+        binding.params_from_dict(prm), pairs), n)
+    binding.res2tac_compute_batch(ctx.handle, pairs, torch.cuda.current_stream().cuda_stream)
+    assert binding.res2tac_last_launch_count(ctx.handle) == 6 * groups
+    single = binding.Stereo(scenes.params(W, H, D, 9, 7, 10, p2, paths, 3))
+    want = [single.compute(*k) for k in keep]
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(want, outs))
+    single.close()
+    ctx.close()
