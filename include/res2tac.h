@@ -283,8 +283,8 @@ int res2tac_autotune(res2tac_t h, const uint8_t* left, const uint8_t* right, int
  *   wta_px     pixels per WTA / right-disparity tile: 64, 128 or 256 (fewer when the tile's sums
  *              would exceed 64 KB, on path planes 29 KB; shear_dpl and shear_cpl have no effect
  *              there)
- * Defaults: row_dpl 2 / 4 / 8 for D <= 64 / <= 128 / larger (8 for D <= 64 on path planes), (16, 1),
- * 128. */
+ * Defaults: row_dpl 2 / 4 / 8 for D <= 64 / <= 128 / larger (8 for D <= 64 on path planes, there 2 in
+ * batches of at most 650 rows in all), (16, 1), 128. */
 typedef struct res2tac_batch_tuning {
   int32_t max_disp, large;
   int32_t row_dpl, shear_dpl, shear_cpl, wta_px;
@@ -302,7 +302,8 @@ int res2tac_get_batch_tuning(res2tac_t h, res2tac_batch_tuning* t);
 /* Autotuner of the batch engine: for the buckets the n pairs fall into (largest total work
  * first; each starts from the defaults) it times the whole batch (res2tac_compute_batch on stream s, median of 3 runs after one
  * warm-up) for each candidate of one setting at a time - row_dpl, then (shear_dpl, shear_cpl),
- * then wta_px - keeping the fastest, and leaves the chosen table in the context. It writes up to
+ * then wta_px - keeping the fastest, and leaves the chosen table in the context, as explicit
+ * settings. Candidates that run the same kernels as another one are not timed. It writes up to
  * cap entries of the buckets it tuned into table (count into *count) and the batch times before
  * and after into *ms_default and *ms_tuned (any of these may be NULL). The pairs' maps are
  * written as by res2tac_compute_batch. Synchronises s; allocates the batch scratch as

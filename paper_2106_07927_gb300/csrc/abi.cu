@@ -746,7 +746,14 @@ int res2tac_autotune_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, re
   std::sort(work.begin(), work.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
   int rc = ensure_engine(h);
   if (rc) return rc;
-  for (const auto& w : work) r2t::batch_set_tune(h->batch, w.second, r2t::batch_default_tune(w.second, r2t::batch_planar_method(h->method)));
+  const bool planar = r2t::batch_planar_method(h->method);
+  int64_t nrows = 0;
+  for (int i = 0; i < n; i++) nrows += pairs[i].height;
+  // each bucket starts from what the defaults run on this batch, so the table names what was timed
+  for (const auto& w : work) {
+    const r2t::BatchTune d = r2t::batch_default_tune(w.second, planar);
+    r2t::batch_set_tune(h->batch, w.second, r2t::batch_resolved_tune(w.second, d, planar, nrows));
+  }
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return fail(RES2TAC_ECUDA, "cudaEventCreate failed");
@@ -758,7 +765,8 @@ int res2tac_autotune_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, re
     const int b = work[wi].second;
     for (int param = 0; param < 3 && !rc; param++) {
       const int ncand = param == 1 ? 2 : 3;
-      r2t::BatchTune keep = r2t::batch_get_tune(h->batch, b, r2t::batch_planar_method(h->method));
+      const r2t::BatchTune keep = r2t::batch_get_tune(h->batch, b, planar);
+      std::vector<r2t::BatchTune> timed(1, keep);
       for (int c = 0; c < ncand && !rc; c++) {
         r2t::BatchTune t = keep;
         if (param == 0) t.row_dpl = (signed char)rows[c];
@@ -767,8 +775,11 @@ int res2tac_autotune_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, re
           t.shear_cpl = (signed char)scpl[c];
         }
         if (param == 2) t.wta_px = (short)wpx[c];
-        if (memcmp(&t, &keep, sizeof(t)) == 0 || !r2t::batch_tune_valid(b, t)) continue;
-        const r2t::BatchTune prev = r2t::batch_get_tune(h->batch, b, r2t::batch_planar_method(h->method));
+        bool same = !r2t::batch_tune_valid(b, t);
+        for (const r2t::BatchTune& o : timed) same |= r2t::batch_tune_same(b, t, o, planar);
+        if (same) continue;
+        timed.push_back(t);
+        const r2t::BatchTune prev = r2t::batch_get_tune(h->batch, b, planar);
         r2t::batch_set_tune(h->batch, b, t);
         const float ms = time_batch(h, pairs, n, st, e0, e1, &rc);
         if (!rc && ms < best) {
@@ -785,7 +796,7 @@ int res2tac_autotune_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, re
   int k = 0;
   for (size_t wi = 0; wi < work.size() && table && k < cap; wi++, k++) {
     const int b = work[wi].second;
-    const r2t::BatchTune v = r2t::batch_get_tune(h->batch, b, r2t::batch_planar_method(h->method));
+    const r2t::BatchTune v = r2t::batch_get_tune(h->batch, b, planar);
     table[k].max_disp = 16 * (b / 2);
     table[k].large = b & 1;
     table[k].row_dpl = v.row_dpl;

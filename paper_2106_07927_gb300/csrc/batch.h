@@ -47,6 +47,12 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
 // Kernel settings per bucket of pairs (tune_bucket: D / 16 and the size class): the defaults,
 // their validity, and the engine's table (set returns -1 for an invalid setting).
 BatchTune batch_default_tune(int bucket, bool planar);
+// The settings t stands for in a batch of that many rows in all: itself, or, for a default on path
+// planes, what such a batch runs, as an explicit setting.
+BatchTune batch_resolved_tune(int bucket, const BatchTune& t, bool planar, int64_t rows);
+// True when the two settings run the same kernels (on path planes the sheared settings have no effect
+// and the selection's tile is capped).
+bool batch_tune_same(int bucket, const BatchTune& a, const BatchTune& b, bool planar);
 bool batch_tune_valid(int bucket, const BatchTune& t);
 int batch_set_tune(BatchEngine* e, int bucket, const BatchTune& t);
 BatchTune batch_get_tune(BatchEngine* e, int bucket, bool planar);

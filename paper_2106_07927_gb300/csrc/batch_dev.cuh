@@ -16,7 +16,8 @@ enum {
 // 64 KB). The persistent sheared kernel holds every setting it may meet inlined, so its settings
 // are kept to the two that cost the most compile time to leave out.
 struct BatchTune {
-  signed char row_dpl, shear_dpl, shear_cpl, pad;
+  signed char row_dpl, shear_dpl, shear_cpl;
+  signed char automatic;  // 1: the default, which a batch on path planes may adapt to its rows
   short wta_px, pad2;
 };
 constexpr int kTuneBuckets = 34;

@@ -231,13 +231,36 @@ BatchTune batch_default_tune(int bucket, bool planar) {
   memset(&t, 0, sizeof(t));
   // On path planes a group has warps enough to hide the row steps' latency, so at D <= 64 the shape
   // with the fewest instructions: 64 x 320x240, D = 64 1357 us with 2 disparities per lane, 1324 with 8
-  // (small batches: see batch_run_planar). At larger D the single pair's: of seven uneven batches
+  // (small batches: see batch_resolved_tune). At larger D the single pair's: of seven uneven batches
   // 8 at D = 128 was up to 2 % slower on three and up to 1.2 % faster on four.
   t.row_dpl = (signed char)(planar && D <= 64 ? 8 : long_dpl_default(D));
+  t.automatic = 1;
   t.shear_dpl = 16;
   t.shear_cpl = 1;
   t.wta_px = 128;
   return t;
+}
+
+// A batch with few rows leaves the row steps' latency open, so its default is the single pair's. us
+// with 2 and with 8 disparities per lane, D = 64: 480 rows (2 x 320x240) 75.2, 77.3, 4 paths 62.0,
+// 70.2; 480 (640x480) 125, 129; 720 (3 x 320x240) 96.6, 90.5; 900 (300x900) 133, 131; 960 (2 x
+// 640x480) 188, 178; 1920 (8 x 320x240) 184, 177. D = 48: 600 (4 x 200x150) 60.2, 61.0; 1200 91.6,
+// 87.1.
+constexpr int64_t kFewRows = 650;
+
+BatchTune batch_resolved_tune(int bucket, const BatchTune& t, bool planar, int64_t rows) {
+  BatchTune r = t;
+  if (t.automatic && planar && rows <= kFewRows)
+    r.row_dpl = (signed char)std::min((int)t.row_dpl, long_dpl_default(16 * (bucket / 2)));
+  r.automatic = 0;
+  return r;
+}
+
+bool batch_tune_same(int bucket, const BatchTune& a, const BatchTune& b, bool planar) {
+  if (a.row_dpl != b.row_dpl) return false;
+  const int D = 16 * (bucket / 2);
+  return planar ? planar_tile_px(D, a.wta_px) == planar_tile_px(D, b.wta_px)
+                : a.shear_dpl == b.shear_dpl && a.shear_cpl == b.shear_cpl && a.wta_px == b.wta_px;
 }
 
 bool batch_tune_valid(int bucket, const BatchTune& t) {
@@ -566,8 +589,11 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
   // groups: pairs of one D and one setting, largest first
   std::vector<int> order((size_t)n);
   std::iota(order.begin(), order.end(), 0);
-  auto tune = [&](int i) -> const BatchTune& {
-    return e->tune[tune_bucket(probs[i].W, probs[i].H, probs[i].D)];
+  int64_t rows = 0;
+  for (int i = 0; i < n; i++) rows += probs[i].H;
+  auto tune = [&](int i) {
+    const int b = tune_bucket(probs[i].W, probs[i].H, probs[i].D);
+    return batch_resolved_tune(b, e->tune[b], true, rows);
   };
   auto alike = [&](int a, int b) {
     return probs[a].D == probs[b].D && lay[a].planes && lay[b].planes &&
@@ -623,11 +649,6 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
     for (int k = 0; k < slots && c == cudaSuccess; k++)
       c = cudaStreamWaitEvent(e->main[k], e->ev_start, 0);
   }
-  // a batch with few rows leaves the row steps' latency open: at most the single pair's setting
-  // (2 x 640x480, D = 64: 254 us with 2 disparities per lane, 260 with 8)
-  int64_t rows = 0;
-  for (int i = 0; i < n; i++) rows += probs[i].H;
-  const bool few = rows <= 1250;
   int total = 0;
   PairGroup pg;
   for (int gi = 0; gi < G && c == cudaSuccess; gi++) {
@@ -650,9 +671,8 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
       at += lay[k].total;
     }
     if (pg.p[0].planar) {
-      const BatchTune& tn = tune(order[g.first]);
-      const int dpl = few ? std::min((int)tn.row_dpl, long_dpl_default(pg.p[0].D)) : tn.row_dpl;
-      c = run_group(pg, mt, dpl, tn.wta_px, st);
+      const BatchTune tn = tune(order[g.first]);
+      c = run_group(pg, mt, tn.row_dpl, tn.wta_px, st);
       total += 6;
     } else {
       int l = 0;

@@ -211,6 +211,8 @@ static cudaError_t launch_planar_wta_t(const Problem& pb, int paths, int T, cuda
                     T);
 }
 
+int planar_tile_px(int D, int wta_px) { return planar_wta_px(D, wta_px); }
+
 static cudaError_t launch_planar_wta(const Problem& pb, const Method& mt, const Tuning& tn,
                                      cudaStream_t s) {
   const int T = planar_wta_px(pb.D, tn.wta_chunk);

@@ -84,6 +84,8 @@ inline cudaError_t launch_agg(void (*kernel)(P...), int grid, int threads, size_
   cfg.numAttrs = dependent ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
+// Pixels per tile of the selection on path planes for the setting wta_chunk / wta_px.
+int planar_tile_px(int D, int wta_px);
 // Settings the plane kernels have (blocks are always one pair of warps): 16 disparities and one chain
 // per lane of the sheared chains, or (8) one chain per warp, one row direction per lane group, costs from the
 // volume of the population-count kernel.

@@ -1,5 +1,6 @@
 """Batch engine: uneven pairs in persistent kernels under a CUDA graph give, per pair, the same
 bits as a single-pair call and as the oracle."""
+import ctypes
 import itertools
 
 import numpy as np
@@ -23,6 +24,44 @@ def _run_batch(h, tensors, shapes):
     binding.res2tac_compute_batch(h, pairs, torch.cuda.current_stream().cuda_stream)
     torch.cuda.synchronize()
     return [binding.u16(o) for o in outs]
+
+
+def _kernels(torch, call):
+    """Names of the kernels that call launches on the current stream, from a capture of it."""
+    cu = ctypes.CDLL("libcuda.so.1")
+
+    def check(rc):
+        assert rc == 0, rc
+    call()
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    graph, n = ctypes.c_void_p(), ctypes.c_size_t()
+    with torch.cuda.stream(s):
+        check(cu.cuStreamBeginCapture_v2(ctypes.c_void_p(s.cuda_stream), 2))  # relaxed
+        try:
+            call()
+        finally:
+            check(cu.cuStreamEndCapture(ctypes.c_void_p(s.cuda_stream), ctypes.byref(graph)))
+    check(cu.cuGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    check(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    names = []
+    for node in nodes:
+        kind = ctypes.c_int()
+        check(cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        if kind.value != 0:  # not a kernel
+            continue
+        # CUDA_KERNEL_NODE_PARAMS: func, 7 x uint32, kernelParams, extra, kern, ctx
+        p = (ctypes.c_uint64 * 16)()
+        check(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), p))
+        name = ctypes.c_char_p()
+        if p[0]:
+            check(cu.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(p[0])))
+        else:
+            check(cu.cuKernelGetName(ctypes.byref(name), ctypes.c_void_p(p[7])))
+        names.append(name.value.decode())
+    check(cu.cuGraphDestroy(graph))
+    return names
 
 
 def _small_batch(seed, n):
@@ -211,4 +250,37 @@ def test_every_batch_tuning_candidate_matches_oracle():
     with pytest.raises(binding.Res2tacError):  # 8 disparities per sheared lane: not a setting
         binding.res2tac_set_batch_tuning(ctx.handle, [binding.res2tac_batch_tuning(64, 0, 2, 8,
                                                                                    1, 128)])
+    ctx.close()
+
+
+def test_explicit_row_setting_runs_on_few_rows():
+    """A batch of few rows adapts the default row_dpl at D <= 64; a setting of the caller's runs as it
+    is, and the autotuner's table names what it timed."""
+    import torch
+    W, H, D = 96, 40, 64
+    L, R, _ = scenes.make_scene("road", 3, W, H, D)
+    ref = oracle.sgm(L, R, D, 9, 7, 10, 120, 8, 3)
+    L, R = torch.from_numpy(L).cuda(), torch.from_numpy(R).cuda()
+    out = torch.empty((H, W), dtype=torch.int16, device="cuda")
+    pairs = [binding.res2tac_pair(L.data_ptr(), R.data_ptr(), W, out.data_ptr(), 2 * W, W, H, D, 0)]
+    ctx = binding.Stereo(scenes.params(64, 64, 64, 9, 7, 10, 120, 8, 3))
+    call = lambda: binding.res2tac_compute_batch(ctx.handle, pairs,
+                                                 torch.cuda.current_stream().cuda_stream)
+    # words per lane and lanes of the row kernel: row_dpl / 2 words, 32 or 8 lanes
+    name = {2: "planar_row_kernelILi1ELi32E", 8: "planar_row_kernelILi4ELi8E"}
+    text = " ".join(_kernels(torch, call))
+    assert name[2] in text and name[8] not in text
+    assert binding.res2tac_get_batch_tuning(ctx.handle, D, 0).row_dpl == 8  # of larger batches
+    binding.res2tac_set_batch_tuning(ctx.handle,
+                                     [binding.res2tac_batch_tuning(D, 0, 8, 16, 1, 128)])
+    text = " ".join(_kernels(torch, call))
+    assert name[8] in text and name[2] not in text
+    assert np.array_equal(binding.u16(out), ref)
+    table, _, _ = binding.res2tac_autotune_batch(ctx.handle, pairs,
+                                                 torch.cuda.current_stream().cuda_stream)
+    text = " ".join(_kernels(torch, call))
+    if table[0].row_dpl in name:
+        assert name[table[0].row_dpl] in text
+    assert table[0].shear_cpl == 1  # no effect on path planes: not a candidate
+    assert np.array_equal(binding.u16(out), ref)
     ctx.close()
