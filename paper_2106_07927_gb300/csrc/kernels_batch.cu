@@ -675,8 +675,20 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
       c = run_group(pg, mt, tn.row_dpl, tn.wta_px, st);
       total += 6;
     } else {
+      // sums in place, the two aggregation kernels one after the other: 803x601, D = 144 563 us
+      // (side by side 491, the persistent kernels 758), 1000x700, D = 256 1151 (1239, 1704),
+      // 1920x1080, D = 64 844 (964, 1155), two of them 1785 (1997, 1791), D = 256 3766 (3722, 4986)
+      const Problem& pb = pg.p[0];
+      const BatchTune& v = e->tune[tune_bucket(pb.W, pb.H, pb.D)];
+      Tuning tn = default_tuning(pb.D);
+      if (!v.automatic) {
+        tn.agg_dpl = v.row_dpl;
+        tn.shear_dpl = v.shear_dpl;
+        tn.shear_cpl = v.shear_cpl;
+        tn.wta_chunk = v.wta_px;
+      }
       int l = 0;
-      c = run_pipeline(pg.p[0], mt, default_tuning(pg.p[0].D), st, &l);
+      c = run_pipeline(pb, mt, tn, st, &l);
       total += l;
     }
   }

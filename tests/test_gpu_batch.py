@@ -284,3 +284,38 @@ def test_explicit_row_setting_runs_on_few_rows():
     assert table[0].shear_cpl == 1  # no effect on path planes: not a candidate
     assert np.array_equal(binding.u16(out), ref)
     ctx.close()
+
+
+def test_pair_without_room_for_planes():
+    """A pair whose planes do not fit the reserved scratch adds its sums in place, with the settings
+    of its bucket."""
+    import torch
+    W, H, D = 1000, 700, 256  # planes: 9 bytes per estimate, 1.6 GB; sums 0.55 + 0.26 GB
+    prm = scenes.params(64, 64, 64, 9, 7, 10, 200, 8, 3)
+    g = torch.Generator("cuda").manual_seed(5)
+    L = torch.randint(0, 256, (H, W), generator=g, device="cuda").to(torch.uint8)
+    R = torch.roll(L, -9, 1).contiguous()
+    out = torch.empty((H, W), dtype=torch.int16, device="cuda")
+    pairs = [binding.res2tac_pair(L.data_ptr(), R.data_ptr(), W, out.data_ptr(), 2 * W, W, H, D, 0)]
+    ctx = binding.Stereo(prm)
+    binding.res2tac_batch_reserve(ctx.handle, binding.res2tac_batch_workspace_bytes(
+        binding.params_from_dict(prm), pairs), 1)
+    call = lambda: binding.res2tac_compute_batch(ctx.handle, pairs,
+                                                 torch.cuda.current_stream().cuda_stream)
+    single = binding.Stereo(scenes.params(W, H, D, 9, 7, 10, 200, 8, 3))
+    want = single.compute(L, R)
+    torch.cuda.synchronize()
+    plain = _kernels(torch, call)
+    assert len(plain) == 6 and not any("planar" in k for k in plain)
+    rows = next(i for i, k in enumerate(plain) if "row" in k)
+    shear = next(i for i, k in enumerate(plain) if "shear" in k)
+    assert torch.equal(out, want)
+    binding.res2tac_set_batch_tuning(ctx.handle,
+                                     [binding.res2tac_batch_tuning(D, 1, 8, 16, 2, 128)])
+    out.fill_(-1)
+    tuned = _kernels(torch, call)
+    torch.cuda.synchronize()
+    assert tuned[rows] == plain[rows] and tuned[shear] != plain[shear]  # two chains per lane
+    assert torch.equal(out, want)
+    single.close()
+    ctx.close()
