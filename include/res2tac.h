@@ -119,7 +119,7 @@ typedef struct res2tac_pair {
  * 128, else 1; wta_chunk 128 (on path planes at most what 29 KB of sums hold).
  * A context on path planes uses them for calls with shear_dpl 8 or 16, shear_cpl 1, row_mode 2,
  * cost_mode 1 and row_cost 1 (agg_warps has no effect there), and adds its sums in place with any
- * other setting. */
+ * other setting, for which the automatic values are those of the other contexts. */
 typedef struct res2tac_tuning {
   int32_t agg_dpl;
   int32_t agg_warps;

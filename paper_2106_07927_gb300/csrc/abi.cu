@@ -415,15 +415,20 @@ int res2tac_get_tuning(res2tac_t h, res2tac_tuning* t) {
 
 int res2tac_set_tuning(res2tac_t h, const res2tac_tuning* t) {
   if (!h || !t) return fail(RES2TAC_EINVAL, "NULL argument");
-  r2t::Tuning n = auto_tuning(h);
-  if (t->agg_dpl) n.agg_dpl = t->agg_dpl;
-  if (t->agg_warps) n.agg_warps = t->agg_warps;
-  if (t->wta_chunk) n.wta_chunk = t->wta_chunk;
-  if (t->shear_dpl) n.shear_dpl = t->shear_dpl;
-  if (t->row_mode) n.row_split = t->row_mode == 2 ? 1 : (t->row_mode == 1 ? 0 : -1);
-  if (t->shear_cpl) n.shear_cpl = t->shear_cpl;
-  if (t->cost_mode) n.cost_mode = t->cost_mode - 1;
-  if (t->row_cost) n.row_cost = t->row_cost - 1;
+  auto with = [&](r2t::Tuning n) {
+    if (t->agg_dpl) n.agg_dpl = t->agg_dpl;
+    if (t->agg_warps) n.agg_warps = t->agg_warps;
+    if (t->wta_chunk) n.wta_chunk = t->wta_chunk;
+    if (t->shear_dpl) n.shear_dpl = t->shear_dpl;
+    if (t->row_mode) n.row_split = t->row_mode == 2 ? 1 : (t->row_mode == 1 ? 0 : -1);
+    if (t->shear_cpl) n.shear_cpl = t->shear_cpl;
+    if (t->cost_mode) n.cost_mode = t->cost_mode - 1;
+    if (t->row_cost) n.row_cost = t->row_cost - 1;
+    return n;
+  };
+  // a setting that leaves the path planes leaves their automatic values too
+  r2t::Tuning n = with(auto_tuning(h));
+  if (h->lay.planes && !r2t::planar_tuning(n)) n = with(r2t::default_tuning(h->p.max_disp));
   if (!r2t::tuning_valid(n, h->p.max_disp))
     return fail(RES2TAC_EINVAL,
                 "tuning (dpl %d, warps %d, chunk %d, shear dpl %d, row mode %d, shear cpl %d, "
@@ -450,7 +455,15 @@ int res2tac_autotune(res2tac_t h, const uint8_t* left, const uint8_t* right, int
           for (int split = 0; split < 2; split++)
             for (int cpl = 1; cpl <= 2; cpl++) {
               r2t::Tuning t{a, w, c, sd, split, cpl, 0, 0};
-              if (r2t::tuning_valid(t, h->p.max_disp)) cands.push_back(t);
+              if (!r2t::tuning_valid(t, h->p.max_disp)) continue;
+              if (h->lay.planes && r2t::planar_tuning(t)) {
+                // there agg_warps has no effect and the tile is capped: one of each kernel
+                if (w != warps[0]) continue;
+                if (c != chunks[0] && r2t::planar_tile_px(h->p.max_disp, c) ==
+                                          r2t::planar_tile_px(h->p.max_disp, c / 2))
+                  continue;
+              }
+              cands.push_back(t);
             }
   if (cands.empty()) return fail(RES2TAC_EINVAL, "no valid tuning");
   cudaEvent_t e0, e1;
@@ -488,13 +501,16 @@ int res2tac_autotune(res2tac_t h, const uint8_t* left, const uint8_t* right, int
   }
   r2t::Problem shape{};
   shape.D = h->p.max_disp;
-  if (!rc && r2t::cost_mma_ok(shape, h->method)) {  // the other cost kernel with the best setting
-    r2t::Tuning t = best_t;
+  // the other cost kernel with the best setting (from path planes, which have no other: with the
+  // automatic settings of the sums)
+  const bool from_planes = h->lay.planes && r2t::planar_tuning(best_t);
+  if (!rc && r2t::cost_mma_ok(shape, h->method)) {
+    r2t::Tuning t = from_planes ? r2t::default_tuning(h->p.max_disp) : best_t;
     t.cost_mode = 1 - t.cost_mode;
     try_tuning(t);
   }
   {  // the row kernel recomputing its costs, with the best setting so far
-    r2t::Tuning t = best_t;
+    r2t::Tuning t = from_planes ? r2t::default_tuning(h->p.max_disp) : best_t;
     t.row_cost = 1;
     if (!rc && r2t::rows_recompute_ok(shape, h->method, t)) try_tuning(t);
   }

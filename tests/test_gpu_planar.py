@@ -106,3 +106,24 @@ def test_reserved_small_batches_run_at_once(n, W, H, D, p2, paths, groups):
     assert all(torch.equal(a, b) for a, b in zip(want, outs))
     single.close()
     ctx.close()
+
+
+def test_settings_off_the_planes_take_the_values_of_the_sums():
+    import torch
+    W, H, D = 200, 60, 128
+    left, right = _pair(3, W, H, D)
+    ref = oracle.sgm(left, right, D, 9, 7, 10, 120, 8, 3)
+    L, R = torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda()
+    st = binding.Stereo(scenes.params(W, H, D, 9, 7, 10, 120, 8, 3))
+    # (shear_dpl, shear_cpl) that a partly given setting ends up with
+    for given, want in ((dict(wta_chunk=64), (8, 1)), (dict(cost_mode=2), (16, 2)),
+                        (dict(row_mode=1), (16, 2)), (dict(row_cost=2), (16, 2)),
+                        (dict(shear_cpl=2), (16, 2)), (dict(shear_dpl=32), (32, 2)),
+                        (dict(cost_mode=2, shear_cpl=1), (16, 1)), (dict(), (8, 1))):
+        binding.res2tac_set_tuning(st.handle, binding.res2tac_tuning(**given))
+        t = binding.res2tac_get_tuning(st.handle)
+        assert (t.shear_dpl, t.shear_cpl) == want, given
+        out = st.compute(L, R)
+        torch.cuda.synchronize()
+        assert np.array_equal(binding.u16(out), ref), given
+    st.close()
