@@ -103,7 +103,8 @@ struct res2tac_ctx {
 
 // The automatic settings of a context.
 static r2t::Tuning auto_tuning(const res2tac_ctx* h) {
-  return h->lay.planes ? r2t::default_planar_tuning(h->p.width, h->p.max_disp, h->p.num_paths)
+  return h->lay.planes ? r2t::default_planar_tuning(h->p.width, h->p.height, h->p.max_disp,
+                                                    h->p.num_paths)
                        : r2t::default_tuning(h->p.max_disp);
 }
 

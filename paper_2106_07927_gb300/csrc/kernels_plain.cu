@@ -131,9 +131,9 @@ Tuning default_tuning(int D) {
   return t;
 }
 
-Tuning default_planar_tuning(int W, int D, int num_paths) {
+Tuning default_planar_tuning(int W, int H, int D, int num_paths) {
   Tuning t = default_tuning(D);
-  t.shear_dpl = planar_shear_dpl(2 * planar_long_pairs(W, num_paths), W);
+  t.shear_dpl = planar_shear_dpl(2 * planar_long_pairs(W, num_paths), W, W > 2 * H);
   t.shear_cpl = 1;
   return t;
 }

@@ -29,7 +29,7 @@ void fork_destroy(Fork* f);
 
 // Default configuration for a disparity count D, and of a pair on path planes.
 Tuning default_tuning(int D);
-Tuning default_planar_tuning(int W, int D, int num_paths);
+Tuning default_planar_tuning(int W, int H, int D, int num_paths);
 // True when the configuration can run a pair with D disparities.
 bool tuning_valid(const Tuning& t, int D);
 

@@ -91,8 +91,9 @@ extern "C" int res2tac_compute_static(const res2tac_params* p, const uint8_t* le
   pb.out_pitch = out_pitch;
   pb.dlf = nullptr;
   int launches = 0;
-  e = r2t::run_pipeline(pb, mt, pb.planar ? r2t::default_planar_tuning(W, D, p->num_paths)
-                                            : r2t::default_tuning(D), (cudaStream_t)s, &launches, nullptr);
+  const r2t::Tuning tn =
+      pb.planar ? r2t::default_planar_tuning(W, H, D, p->num_paths) : r2t::default_tuning(D);
+  e = r2t::run_pipeline(pb, mt, tn, (cudaStream_t)s, &launches, nullptr);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return reject(RES2TAC_ECUDA, "res2tac_compute_static: launch failed: %s",

@@ -86,6 +86,13 @@ constexpr int kRowStages = 4, kRowChunk = 8;
 __host__ __device__ inline int planar_ring_smem(int D, int lpl) {
   return 2 * kRowStages * kRowChunk * (32 / lpl) * D;
 }
+// Byte of a pixel where the lane with number lig of a chain starts, NW words a lane (0 for a lane past
+// the chain's words, whose reads are not used).
+__host__ __device__ inline int planar_lane_at(int lig, int NW, int D) {
+  return lig < D / (2 * NW) ? lig * 2 * NW : 0;
+}
+// Pixel at which the two directions of a row meet when they share a plane.
+__host__ __device__ inline int planar_row_mid(int W) { return (W / 2) & ~(kRowChunk - 1); }
 // Warps of one direction: 32 / lanes rows each.
 __host__ __device__ inline int planar_row_warps(int H, int lpl) {
   const int cpw = 32 / lpl;
@@ -212,7 +219,7 @@ __device__ __forceinline__ void planar_rows(const Problem& pb, const Method& mt,
   const int y = y0 + c;
   LongChain<NW, LPL, FULL> chain(lane, D);
   const bool valid = y < pb.H, active = valid && chain.owns;
-  const int at = chain.owns ? lig * 2 * NW : 0;  // the lane's bytes of a pixel (else: never used)
+  const int at = planar_lane_at(lig, NW, D);
   const bool paired = planar_paired(mt);
   const int64_t row = (int64_t)(valid ? y : 0) * W * D;
   const uint32_t slot_bytes = (uint32_t)(CPW * G * D);
@@ -293,7 +300,7 @@ __device__ __forceinline__ void planar_rows(const Problem& pb, const Method& mt,
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
   };
-  const int mid = (W / 2) & ~(G - 1);
+  const int mid = planar_row_mid(W);
   if (paired) {
     walk(BACK ? mid : 0, BACK ? W : mid, std::false_type());
     __syncthreads();
@@ -312,6 +319,8 @@ __device__ __forceinline__ void planar_rows(const Problem& pb, const Method& mt,
 //   adjacent pixels, so both are contiguous over the warp. The fewest instructions per estimate.
 // - planar_long: one chain per warp, as the row paths. The shortest step, for small images.
 constexpr int kPlanarRing = 8;
+constexpr int kShearGroup = 2;                          // steps between two tests for a wrap
+constexpr int kShearAhead = kPlanarRing - kShearGroup;  // steps from a cost copy to its use
 __host__ __device__ inline int planar_shear_smem() { return kPlanarRing * 1024; }  // of one warp
 // Pairs of warps: the two opposite directions of a group of adjacent chains, or of one chain.
 __host__ __device__ inline int planar_shear_pairs(int W, int D, int num_paths) {
@@ -325,14 +334,19 @@ __host__ __device__ inline int planar_long_pairs(int W, int num_paths) {
 __host__ __device__ inline int planar_long_words(int D) { return D <= 64 ? 1 : (D <= 128 ? 2 : 4); }
 // Shape of a launch over pairs of that many chains in all (setting shear_dpl): 8 for one chain per
 // warp, 16 otherwise. The line lies where the warps of the 16-disparity shape leave most schedulers
-// with one or none, so that a step's latency decides: us per call with one chain per warp and with
-// 16 disparities per lane, 8 paths: 160x120 D=32 (960 chains) 38, 44; 320x240 D=64 (1920) 54, 66;
-// 413x307 D=48 (2478) 83, 80; 640x480 D=64 (3840) 138, 132; 1242x375 D=128 (7452) 280, 262.
+// with one or none, so that a step's latency decides, unless the rows' chains, which run beside, are
+// the longer ones (W > 2 H) and only the work counts. us per call with one chain per warp and with 16
+// disparities per lane, 8 paths: 160x120, D = 32 (960 chains) 38, 44; 320x375, D = 64 (1920) 65, 77, D
+// = 128 84, 94, D = 224 137, 128; 413x307, D = 48 (2478) 83, 80; 640x480, D = 64 (3840) 138, 132;
+// W > 2 H: 320x120, D = 32 (1920) 43, 40, D = 256 65, 53; 4 paths: 413x375, D = 144 (826) equal;
+// 640x375, D = 64 (1280) 0.90 of the other, D = 144 147, 123; 1000x375, D = 128 (2000) 148, 146, D =
+// 256 265, 247. Tall pairs of large D would gain from it past the line too (413x900, D = 256, 2478
+// chains 397, 528); D between 160 and 240 lose up to 8 % of a call at it (320x375).
 // wmin: the smallest width among them (a chunk of the one-chain-per-warp walk wraps around the image
-// edge at most once).
+// edge at most once); flat: one of them has W > 2 H.
 constexpr int64_t kLongChains = 2200;
-inline int planar_shear_dpl(int64_t chains, int wmin) {
-  return wmin >= kRowChunk && chains <= kLongChains ? 8 : 16;
+inline int planar_shear_dpl(int64_t chains, int wmin, bool flat) {
+  return wmin >= kRowChunk && !flat && chains <= kLongChains ? 8 : 16;
 }
 
 // Minimum over the NL lanes of a group of a value whose halves are equal. Any NL: rotations by
@@ -384,7 +398,7 @@ template <int NL>
 __device__ __forceinline__ void planar_shear(const Problem& pb, const Method& mt, int item,
                                              bool back, uint8_t* ring) {
   constexpr int NP = 8, LB = 16, D = LB * NL, CH = 32 / NL;
-  constexpr int GS = 2, KS = kPlanarRing, PF = KS - GS;
+  constexpr int GS = kShearGroup, KS = kPlanarRing, PF = kShearAhead;
   constexpr int SLOT = 1024, OTHER = 512;  // costs, then the other direction's U
   const int lane = threadIdx.x & 31, c = lane / NL, lig = lane - c * NL;
   const bool in = c < CH;
@@ -553,7 +567,7 @@ __device__ __forceinline__ void planar_long(const Problem& pb, const Method& mt,
   const int dy = back ? -1 : 1, dx = back ? -sh : sh;
   const int ystart = back ? H - 1 : 0;
   LongChain<NW, 32, FULL> chain(lane, D);
-  const int at = chain.owns ? lane * 2 * NW : 0;  // the lane's bytes of a pixel (else: never used)
+  const int at = planar_lane_at(lane, NW, D);
   const uint32_t P1P1 = (uint32_t)mt.P1 * 0x10001u, P2P2 = (uint32_t)mt.P2 * 0x10001u;
   const uint32_t slot_bytes = (uint32_t)(G * D);
   const uint32_t other = kRowStages * slot_bytes;  // the other direction's U behind the costs

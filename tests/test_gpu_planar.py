@@ -110,7 +110,7 @@ def test_reserved_small_batches_run_at_once(n, W, H, D, p2, paths, groups):
 
 def test_settings_off_the_planes_take_the_values_of_the_sums():
     import torch
-    W, H, D = 200, 60, 128
+    W, H, D = 200, 110, 128
     left, right = _pair(3, W, H, D)
     ref = oracle.sgm(left, right, D, 9, 7, 10, 120, 8, 3)
     L, R = torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda()

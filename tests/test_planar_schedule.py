@@ -1,18 +1,42 @@
 """Host models of the walks on path planes (csrc/planar.cuh): every cost copy and every store of a
 sheared chain, with its restarts, against the chain definition; the row walk's chunks; and the
-scan ranges of the selection's diagonals against the definition of D^R."""
+scan ranges of the selection's diagonals against the definition of D^R. The constants, ring sizes,
+tiles, lane offsets and the rule for the sheared chains' shape are the header's own, printed by
+planar_host.cu."""
 import itertools
+import os
+import subprocess
 
 import pytest
+
+from paper_2106_07927_gb300 import build
 
 NEVER = 1 << 30
 
 
-def _walk(W, H, kind, j, paired):
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    """{first word: {key numbers: last number(s)}} of what planar_host.cu prints."""
+    exe = str(tmp_path_factory.mktemp("host") / "planar_host")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "planar_host.cu")
+    subprocess.run([build.nvcc(), *build.ARCH, "-std=c++17", "-o", exe, src], check=True)
+    keys = {"const": 0, "shear_smem": 0, "mid": 1, "ring": 2, "tile": 2, "words": 1, "at": 3,
+            "lanes": 2, "shape": 3}
+    out = {}
+    for line in subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split("\n"):
+        if line:
+            word, *v = line.split()
+            v = tuple(map(int, v))
+            k = keys[word]
+            out.setdefault(word, {})[v[:k]] = v[k:] if len(v) - k > 1 else v[k]
+    return out
+
+
+def _walk(W, H, kind, j, paired, GS, PF):
     """(copies, stores, restarts) of one chain alone in its warp, pixel by pixel, as the kernel's
     two pointers and its fast and general groups of GS steps make them, in one part or (directions
-    that share a plane) in two; copies are listed by the step that uses them."""
-    GS, PF = 2, 6  # steps of a group, and between a cost copy and its use
+    that share a plane) in two; copies are listed by the step that uses them. GS: steps of a group,
+    PF: steps between a cost copy and its use."""
     sh = 0 if kind < 2 else (1 if kind < 4 else -1)
     back = kind & 1
     dy, dx = (-1, -sh) if back else (1, sh)
@@ -70,9 +94,8 @@ def _walk(W, H, kind, j, paired):
     return copies, stores, restarts
 
 
-def _long_walk(W, H, kind, j, paired):
-    """The same of the walk with one chain per warp: 8-step chunks, one cursor per step of a chunk."""
-    G = 8
+def _long_walk(W, H, kind, j, paired, G):
+    """The same of the walk with one chain per warp: chunks of G steps, one cursor per step."""
     sh = 0 if kind < 2 else (1 if kind < 4 else -1)
     back = kind & 1
     dy, dx = (-1, -sh) if back else (1, sh)
@@ -112,7 +135,9 @@ def _long_walk(W, H, kind, j, paired):
 
 
 @pytest.mark.parametrize("kind", range(6))
-def test_sheared_walk_on_planes(kind):
+def test_sheared_walk_on_planes(host, kind):
+    _, G, ring, GS, PF = host["const"][()]
+    assert ring & (ring - 1) == 0 and GS + PF <= ring
     for W, H in itertools.product((1, 2, 3, 5, 8, 13, 40), (1, 2, 5, 6, 7, 8, 9, 14, 15, 33, 100)):
         sh = 0 if kind < 2 else (1 if kind < 4 else -1)
         for j in range(W):
@@ -121,18 +146,19 @@ def test_sheared_walk_on_planes(kind):
             entry = (0 if sh > 0 else W - 1) if not kind & 1 else (W - 1 if sh > 0 else 0)
             starts = [t for t, p in enumerate(want) if sh and t and p % W == entry]
             for paired in (False, True):
-                got = _walk(W, H, kind, j, paired)
+                got = _walk(W, H, kind, j, paired, GS, PF)
                 assert got == (want, want, starts), (W, H, j, paired)
-                if W >= 8:
-                    got = _long_walk(W, H, kind, j, paired)
+                if W >= G:
+                    got = _long_walk(W, H, kind, j, paired, G)
                     assert got == (want, want, starts), (W, H, j, paired, "long")
 
 
 @pytest.mark.parametrize("back", [False, True])
-def test_row_walk_chunks(back):
-    G = 8
+def test_row_walk_chunks(host, back):
+    G = host["const"][()][1]
     for W, paired in itertools.product(range(1, 60), (False, True)):
-        mid = (W // 2) & ~(G - 1)
+        mid = host["mid"][(W,)]
+        assert mid % G == 0
         got, met = [], [0, 0]
         for ph in range(2 if paired else 1):
             low = paired and (ph == 0) != back
@@ -182,24 +208,26 @@ def test_selection_scans_every_sum_once(W, D, T):
 
 
 @pytest.mark.parametrize("D", range(16, 257, 16))
-def test_ring_accesses_stay_inside(D):
+def test_ring_accesses_stay_inside(host, D):
     # shared-memory reads and copies of the row walk and of the walk with one chain per warp, in the
-    # bytes planar_ring_smem gives one warp: 2 x 4 slots of 8 pixels of each chain
-    shapes, G = [(1 if D <= 64 else 2 if D <= 128 else 4, 32)], 8  # one chain per warp
+    # bytes planar_ring_smem gives one warp: costs and the other direction's U, stages of G pixels
+    stages, G = host["const"][()][:2]
+    assert stages & (stages - 1) == 0
+    shapes = [(host["words"][(D,)], 32)]  # one chain per warp
     for dpl in (2, 4, 8):
-        if D // dpl <= 32:
-            lanes = 8
-            while lanes < D // dpl:
-                lanes *= 2
-            shapes.append((dpl // 2, lanes))
+        if (D, dpl) in host["lanes"]:
+            shapes.append((dpl // 2, host["lanes"][(D, dpl)]))
     for nw, lpl in shapes:
         cpw = 32 // lpl
-        size = 2 * 4 * G * cpw * D
-        slot_bytes, other = cpw * G * D, 4 * cpw * G * D
+        assert 2 * nw * lpl >= D
+        size = host["ring"][(D, lpl)]
+        slot_bytes = cpw * G * D
+        other = stages * slot_bytes
         for lane in range(32):
             c, lig = lane // lpl, lane % lpl
-            at = lig * 2 * nw if lig < D // (2 * nw) else 0
-            for stage in (0, 3):
+            at = host["at"][(D, nw, lig)]
+            assert at == (lig * 2 * nw if lig * 2 * nw < D else 0)
+            for stage in range(stages):
                 base = c * G * D + stage * slot_bytes + other
                 assert base + (G - 1) * D + at + 2 * nw <= size
                 for v in range(nw):
@@ -208,3 +236,17 @@ def test_ring_accesses_stay_inside(D):
                         assert base + 16 * i + 16 <= size
         # every piece of a chunk is copied by some lane
         assert {lig + lpl * v for lig in range(lpl) for v in range(nw)} >= set(range(G * D // 16))
+
+
+def test_selection_tiles(host):
+    # whole blocks of 32 pixels, no more than asked for, and the sums with the keys behind them
+    for (D, T), (px, smem) in host["tile"].items():
+        assert px % 32 == 0 and 32 <= px <= T
+        assert smem == px * (D // 2 + 1) * 4 + (px + D) * 8 <= 32 * 1024
+
+
+def test_shape_of_the_sheared_chains(host):
+    # one chain per warp on small images whose rows are not the longer walk
+    assert host["shape"] == {(160, 120, 8): 8, (320, 240, 8): 8, (320, 120, 8): 16,
+                             (413, 307, 8): 16, (1000, 375, 4): 16, (640, 375, 4): 8,
+                             (7, 9, 8): 16, (8, 9, 8): 8}
