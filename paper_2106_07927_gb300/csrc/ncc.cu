@@ -41,16 +41,26 @@ inline size_t ncc_smem(int n, int TY) {
 }
 
 // Output rows of a block. A block computes n - 1 rows of dot products more than it outputs, so long
-// bands are cheaper, but the last wave of blocks should be full: the band with the least waves x
-// (TY + n - 1 rows + about 4 rows' worth of staging). Stage us, 9 x 9, against bands of 32 rows: 640
-// x 480, D = 64 87 -> 77; 1242 x 375, D = 128 189 -> 185; 1920 x 1080, D = 256 1347 -> 1309; 5 x 5, 350
-// x 260, D = 112 51 -> 44.
+// bands are cheaper, but the last wave of blocks should be full.
+// 9 x 9: the band with the least waves x (TY + n - 1 rows + about 4 rows' worth of staging). us per
+// call against bands of 32 rows: 640 x 480, D = 64 227 -> 215; 1242 x 375, D = 128 443 -> 440; 1920 x
+// 1080, D = 256 4811 -> 4770.
+// 5 x 5: four rows more cost little, so short bands, which even out the last wave: the shortest of 16
+// to 32 rows with which all blocks run at once, else 20, or 28 past 8 waves of blocks. Against bands
+// of 32 rows and of the 9 x 9 rule: 350 x 260, D = 112 142, 133 -> 133; 640 x 480, D = 64 206.5, 204.7
+// -> 204.9; 1242 x 375, D = 128 414, 421 -> 406; 1300 x 700, D = 64 430, 435 -> 427; 1920 x 1080, D =
+// 256 4596, 4591 -> 4583.
 int ncc_band(int W, int H, int D, int n) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t fit = (int64_t)std::max(sms, 1) * (n == 5 ? 4 : 3);  // blocks at a time
   const int64_t ntx = (W + ncc_tx(D) - 1) / ncc_tx(D);
+  if (n == 5) {
+    for (int TY = 16; TY <= 32; TY++)
+      if (ntx * ((H + TY - 1) / TY) <= fit) return TY;
+    return ntx * ((H + 19) / 20) <= 8 * fit ? 20 : 28;
+  }
   int best = 16;
   int64_t least = INT64_MAX;
   for (int TY = 16; TY <= kNccMaxTY; TY++) {
