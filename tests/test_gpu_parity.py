@@ -332,7 +332,11 @@ def test_ncc_tiny_random_shapes(seed):
     _assert_same(left, right, prm)
 
 
-@pytest.mark.parametrize("W,H,D,n", [(200, 37, 64, 5), (97, 61, 128, 9), (130, 33, 256, 9)])
+# and the bands of the cost kernel, with a last band of one or a few rows: 5 x 5 of 18, 20 and 28 rows,
+# 9 x 9 of 44
+@pytest.mark.parametrize("W,H,D,n", [(200, 37, 64, 5), (97, 61, 128, 9), (130, 33, 256, 9),
+                                     (350, 253, 112, 5), (640, 481, 64, 5), (1210, 337, 256, 5),
+                                     (640, 480, 64, 9)])
 def test_ncc_ragged_tiles(W, H, D, n):
     left, right, _ = scenes.make_scene("road", W + H + n, W, H, D)
     _assert_same(left, right, scenes.params(W, H, D, n, n, 90, 880, 8, 3 | NCC))
