@@ -650,6 +650,7 @@ int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res
     pb.in_pitch = q.in_pitch;
     pb.disp = q.disp;
     pb.out_pitch = q.out_pitch;
+    pb.fault = reinterpret_cast<unsigned*>(h->scratch + h->lay.fault);
     probs[i] = pb;
   }
   int launches = 0;

@@ -52,7 +52,9 @@ struct Problem {
 // constant true and compiles away.
 // Sites: 1 row-kernel cost load, 2 row-kernel add into S, 3 sheared-kernel cost copy, 4 / 5
 // sheared-kernel bulk add (run before / after a wrap), 6 WTA staging copy of S, 7 WTA store of D^L.
-// (planes: 3 also the own-lane cost copies, 2 and 4 the stores of U)
+// Planes: 1 and 3 copies of the costs and of the other direction's U, 2 and 4 stores of U (rows,
+// sheared), 6 the selection's loads of the cost and the planes, 7 its stores of D^L (and the sub-pixel
+// one), 9 its D^R keys. The record is the context's, for batches too.
 // Site 8 is recorded in every build: a block of the tensor-core cost kernel whose MMAs did not
 // complete within its poll limit (it stores no cost).
 #ifdef RES2TAC_CHECK_BOUNDS

@@ -667,6 +667,7 @@ int batch_run_planar(BatchEngine* e, const Problem* probs, int n, const Method& 
       pb.in_pitch = q.in_pitch;
       pb.disp = q.disp;
       pb.out_pitch = q.out_pitch;
+      pb.fault = q.fault;
       pb.dlf = nullptr;
       at += lay[k].total;
     }

@@ -743,11 +743,15 @@ __device__ __forceinline__ void planar_wta_tile(const Problem& pb, int paths, in
     // exact i / ppx for i < 2^16 (2^32 / 1 does not fit: D = 16 takes i itself)
     const uint32_t inv = (uint32_t)((0xFFFFFFFFull + ppx) / ppx);
     for (int i = threadIdx.x; i < n * ppx; i += blockDim.x) {
-      uint4 cw, u[R];
-      cw = __ldcs(reinterpret_cast<const uint4*>(cost) + i);
+      uint4 cw = make_uint4(0, 0, 0, 0), u[R];
+      if (R2T_CHECKED(pb, cost + 16 * (int64_t)i, 16, pb.cost, pb.plane, 6))
+        cw = __ldcs(reinterpret_cast<const uint4*>(cost) + i);
 #pragma unroll
-      for (int r = 0; r < R; r++)
-        u[r] = __ldcs(reinterpret_cast<const uint4*>(pl + r * pb.plane) + i);
+      for (int r = 0; r < R; r++) {
+        u[r] = make_uint4(0, 0, 0, 0);
+        if (R2T_CHECKED(pb, pl + r * pb.plane + 16 * (int64_t)i, 16, pb.agg, R * pb.plane, 6))
+          u[r] = __ldcs(reinterpret_cast<const uint4*>(pl + r * pb.plane) + i);
+      }
       const int px = ppx == 1 ? i : (int)__umulhi((uint32_t)i, inv), q = i - px * ppx;
       uint32_t* o = S + px * pitch + 4 * q;
       auto sum = [&](uint32_t cword, auto&& get, int j) {
@@ -797,7 +801,7 @@ __device__ __forceinline__ void planar_wta_tile(const Problem& pb, int paths, in
           const int s0 = s[0] >> 4, a = (s[-1] >> 4) - s0, b = (s[1] >> 4) - s0;
           v = __fadd_rn(v, __fdiv_rn((float)(a - b), (float)(2 * (a + b))));
         }
-        pb.dlf[p] = v;
+        if (R2T_CHECKED(pb, pb.dlf + p, 4, pb.dlf, 4 * (int64_t)W * pb.H, 7)) pb.dlf[p] = v;
       }
     } else {
       const int j = i - n, t = j - (D - 1);  // relative to x0
@@ -833,6 +837,7 @@ __device__ __forceinline__ void planar_wta_tile(const Problem& pb, int paths, in
     if (x < 0) continue;
     const uint32_t k = min(klo[j], j + 1 < nd ? khi[j + 1] : 0xFFFFFFFFu);
     if (k >= 0xFFF00u) continue;
+    if (!R2T_CHECKED(pb, pb.kr + rowbase + x, 4, pb.kr, 4 * (int64_t)W * pb.H, 9)) continue;
     if (x >= x0 && min(x + D - 1, W - 1) < x0 + n)
       pb.kr[rowbase + x] = k;
     else

@@ -24,7 +24,9 @@ def test_range_checks_pass_on_tiny_shapes(check_lib):
     rng = np.random.default_rng(77)
     cases = [(1, 1, 16), (5, 3, 16), (17, 9, 32), (33, 20, 48), (70, 13, 64), (9, 40, 128),
              (130, 7, 144), (40, 31, 256)]
-    for (W, H, D), (p2, paths) in zip(cases, itertools.cycle(((120, 8), (16384, 8), (90, 4)))):
+    # one plane per two directions and one per direction, 16-bit and 32-bit sums
+    methods = ((120, 8), (16384, 8), (90, 4), (200, 8), (255, 4), (880, 8))
+    for (W, H, D), (p2, paths) in itertools.product(cases, methods):
         left = rng.integers(0, 256, (H, W)).astype(np.uint8)
         right = rng.integers(0, 256, (H, W)).astype(np.uint8)
         prm = scenes.params(W, H, D, 9, 7, 10, p2, paths, 3)
@@ -41,4 +43,36 @@ def test_range_checks_pass_on_tiny_shapes(check_lib):
             checked, site, off = binding.res2tac_bounds_status(st.handle)
             assert site == 0, (W, H, D, sdpl, mode, cpl, site, off)
             assert np.array_equal(binding.u16(out), ref), (W, H, D, sdpl, mode, cpl)
+        if p2 <= 255:  # the selection's sub-pixel map
+            binding.res2tac_set_tuning(st.handle, binding.res2tac_tuning())
+            st.compute_subpixel(L, R)
+            torch.cuda.synchronize()
+            assert binding.res2tac_bounds_status(st.handle)[1] == 0, (W, H, D, p2, "subpixel")
         st.close()
+
+
+@pytest.mark.parametrize("p2,paths", [(120, 8), (200, 8), (200, 4), (880, 8), (16384, 8)])
+def test_range_checks_pass_in_batches(check_lib, p2, paths):
+    import torch
+    rng = np.random.default_rng(78)
+    shapes = [(1, 1, 16), (5, 3, 16), (33, 20, 48), (31, 24, 48), (9, 40, 128), (130, 7, 144),
+              (40, 31, 256), (300, 12, 64)] + [(40, 9, 32)] * 35
+    prm = scenes.params(64, 64, 64, 9, 7, 10, p2, paths, 3)
+    st = binding.Stereo(prm)
+    keep, pairs, refs = [], [], []
+    for W, H, D in shapes:
+        left = rng.integers(0, 256, (H, W)).astype(np.uint8)
+        right = rng.integers(0, 256, (H, W)).astype(np.uint8)
+        L, R = torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda()
+        o = torch.full((H, W), -1, dtype=torch.int16, device="cuda")
+        keep.append((L, R, o))
+        pairs.append(binding.res2tac_pair(L.data_ptr(), R.data_ptr(), W, o.data_ptr(), 2 * W, W, H,
+                                          D, 0))
+        refs.append(oracle.sgm(left, right, D, 9, 7, 10, p2, paths, 3))
+    binding.res2tac_compute_batch(st.handle, pairs, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    checked, site, off = binding.res2tac_bounds_status(st.handle)
+    assert (checked, site) == (1, 0), (site, off)
+    for (_, _, o), ref in zip(keep, refs):
+        assert np.array_equal(binding.u16(o), ref)
+    st.close()
