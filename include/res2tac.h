@@ -137,10 +137,21 @@ typedef struct res2tac_tuning {
  * Where p2 <= 255, the cost is the census, the scratch stays below 32 GB (W H D below 2^32) and at
  * least half of the device's memory stays free with it, the context keeps the paths' terms as byte
  * planes instead of one volume of sums, which is faster, with identical results: 1 + num_paths / 2
- * bytes per W*H*D with 2 p2 <= 255, else 1 + num_paths (3 with sums, 5 with 32-bit ones), and 4 B
- * more per pixel. Otherwise it allocates res2tac_workspace_bytes.
+ * bytes per W*H*D with 2 p2 <= 255, else 1 + num_paths (3 with sums), and 4 B more per pixel.
+ * Otherwise it allocates res2tac_workspace_bytes. So contexts whose res2tac_workspace_bytes add up
+ * to the device's memory need not all fit: a caller that admits contexts by that number creates
+ * them with res2tac_create_compact, or reads what each one took (res2tac_context_bytes).
  * Returns RES2TAC_EINVAL for invalid parameters, RES2TAC_ENOMEM if the scratch does not fit. */
 int res2tac_create(const res2tac_params* p, res2tac_t* out);
+
+/* As res2tac_create, without memory for path planes: the context takes at most
+ * res2tac_workspace_bytes, and its batch scratch at most what res2tac_batch_workspace_bytes or
+ * res2tac_batch_reserve ask for. Identical results. */
+int res2tac_create_compact(const res2tac_params* p, res2tac_t* out);
+
+/* Device bytes the context holds now: its scratch, staging and rectification maps and its batch
+ * scratch (0 for NULL). */
+size_t res2tac_context_bytes(res2tac_t h);
 
 /* Runs the whole pipeline of Sec. 2.1 on one rectified pair, asynchronously on stream s:
  * census (Sec. 2.2.1) -> Hamming cost, Eq. (image_matching) -> SGM aggregation over num_paths
@@ -245,9 +256,10 @@ int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res
 int res2tac_debug_outputs(res2tac_t h, uint8_t* cost, uint16_t* agg, uint16_t* dl, uint16_t* dr,
                           uint8_t* mask, res2tac_stream_t s);
 
-/* Device bytes a context for *p needs (0 if *p is invalid); for admission control. It takes more,
- * for path planes, only where at least half of the device's memory stays free (see
- * res2tac_create). */
+/* Device bytes a context for *p needs (0 if *p is invalid), and the most that
+ * res2tac_create_compact takes; for admission control. res2tac_create takes more, for path planes,
+ * where at least half of the device's memory stays free with it: then up to 1.7 (2 p2 <= 255) or 3
+ * times as much. */
 size_t res2tac_workspace_bytes(const res2tac_params* p);
 
 /* Device bytes a batch of n pairs needs on top of the context (0 if a pair is invalid); see

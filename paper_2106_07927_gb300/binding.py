@@ -30,7 +30,7 @@ EXPORTS = (
     "res2tac_get_tuning", "res2tac_set_tuning", "res2tac_autotune", "res2tac_last_launch_count",
     "res2tac_destroy", "res2tac_strerror", "res2tac_last_error", "res2tac_set_profiling",
     "res2tac_stage_times",
-    "res2tac_batch_reserve",
+    "res2tac_batch_reserve", "res2tac_create_compact", "res2tac_context_bytes",
     "res2tac_compute_static",
     "res2tac_compute_subpixel", "res2tac_debug_subpixel",
     "res2tac_rectify", "res2tac_set_rectification", "res2tac_compute_raw",
@@ -99,6 +99,8 @@ def load(path: str | None = None):
     PP = ctypes.POINTER(res2tac_params)
     sig = {
         "res2tac_create": (ctypes.c_int, [PP, ctypes.POINTER(ctypes.c_void_p)]),
+        "res2tac_create_compact": (ctypes.c_int, [PP, ctypes.POINTER(ctypes.c_void_p)]),
+        "res2tac_context_bytes": (S, [P]),
         "res2tac_compute": (ctypes.c_int, [P, P, P, I64, P, I64, P]),
         "res2tac_compute_host": (ctypes.c_int, [P, P, P, I64, P, I64, P]),
         "res2tac_compute_batch": (ctypes.c_int, [P, ctypes.POINTER(res2tac_pair), I32, P]),
@@ -182,6 +184,16 @@ def res2tac_create(params: res2tac_params) -> int:
     h = ctypes.c_void_p()
     _check(load().res2tac_create(ctypes.byref(params), ctypes.byref(h)))
     return h.value
+
+
+def res2tac_create_compact(params: res2tac_params) -> int:
+    h = ctypes.c_void_p()
+    _check(load().res2tac_create_compact(ctypes.byref(params), ctypes.byref(h)))
+    return h.value
+
+
+def res2tac_context_bytes(h: int) -> int:
+    return int(load().res2tac_context_bytes(h))
 
 
 def res2tac_compute(h: int, left: int, right: int, in_pitch: int, disp: int, out_pitch: int,
@@ -344,9 +356,9 @@ class Stereo:
     """One context bound to torch CUDA tensors: torch supplies device memory and the stream only;
     all computation happens in the library's kernels."""
 
-    def __init__(self, params):
+    def __init__(self, params, compact=False):
         self.params = params if isinstance(params, res2tac_params) else params_from_dict(params)
-        self.handle = res2tac_create(self.params)
+        self.handle = (res2tac_create_compact if compact else res2tac_create)(self.params)
 
     def close(self):
         if self.handle:

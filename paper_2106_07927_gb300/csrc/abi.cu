@@ -96,6 +96,7 @@ struct res2tac_ctx {
   int last_planar;     // the last call left path planes (else one volume of sums)
   r2t::BatchEngine* batch;
   int batch_reserved;  // the batch scratch was sized by res2tac_batch_reserve
+  int compact;         // no memory for path planes beyond what the sums take
   int profiling;
   cudaEvent_t ev[8];  // stage boundaries of the last profiled compute (8 with the exact check)
   r2t::Fork fork;     // second stream for the concurrent aggregation kernels
@@ -130,7 +131,7 @@ size_t res2tac_workspace_bytes(const res2tac_params* p) {
          npx * 2 + 1024;
 }
 
-int res2tac_create(const res2tac_params* p, res2tac_t* out) {
+static int create(const res2tac_params* p, res2tac_t* out, bool compact) {
   if (!out) return fail(RES2TAC_EINVAL, "out is NULL");
   *out = nullptr;
   if (const char* why = params_error(p)) return fail(RES2TAC_EINVAL, "res2tac_create: %s", why);
@@ -139,6 +140,7 @@ int res2tac_create(const res2tac_params* p, res2tac_t* out) {
   memset(h, 0, sizeof(*h));
   h->p = *p;
   h->method = method_of(*p);
+  h->compact = compact;
   cudaError_t e = cudaGetDevice(&h->device);
   if (e != cudaSuccess) {
     delete h;
@@ -147,7 +149,8 @@ int res2tac_create(const res2tac_params* p, res2tac_t* out) {
   // path planes only where half of the device's memory stays free with them
   const size_t npx = (size_t)p->width * p->height;
   size_t free_b = 0, total_b = 0;
-  h->lay = r2t::layout_single(p->width, p->height, p->max_disp, h->method);
+  h->lay = r2t::layout_single(p->width, p->height, p->max_disp, h->method,
+                              compact ? 0 : r2t::kPlanarBytes);
   if (h->lay.planes && (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
                         h->lay.total + 4 * npx + total_b / 2 > free_b ||
                         cudaMalloc(&h->scratch, h->lay.total) != cudaSuccess)) {
@@ -168,6 +171,17 @@ int res2tac_create(const res2tac_params* p, res2tac_t* out) {
   }
   *out = h;
   return RES2TAC_OK;
+}
+
+int res2tac_create(const res2tac_params* p, res2tac_t* out) { return create(p, out, false); }
+
+int res2tac_create_compact(const res2tac_params* p, res2tac_t* out) { return create(p, out, true); }
+
+size_t res2tac_context_bytes(res2tac_t h) {
+  if (!h) return 0;
+  const size_t npx = (size_t)h->p.width * h->p.height;
+  return h->lay.total + 2 * align_up(npx * 2, 256) + (h->maps ? 16 * npx : 0) +
+         r2t::batch_bytes(h->batch);
 }
 
 void res2tac_destroy(res2tac_t h) {
@@ -597,7 +611,7 @@ size_t res2tac_batch_workspace_bytes(const res2tac_params* p, const res2tac_pair
 // planes at once instead of a few pairs at a time: the planes of everything that fits `total` (2
 // to 8 bytes per estimate against the sums' 2, of 3 with the cost), at most kBatchExtra.
 static size_t batch_extra(res2tac_t h, size_t total) {
-  const int planes = r2t::method_planes(h->method);
+  const int planes = h->compact ? 0 : r2t::method_planes(h->method);
   return planes > 2 ? std::min(r2t::kBatchExtra, total / 3 * (planes - 2) + 65536) : 0;
 }
 
@@ -632,7 +646,7 @@ int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res
       return fail(RES2TAC_EINVAL, "pair %d: bad pitch", i);
     offs[i] = total;
     total += layout_for(q.width, q.height, q.max_disp, wide).total;
-    if (planar && !h->batch_reserved)  // grown on demand: room for the planes of a lone pair
+    if (planar && !h->batch_reserved && !h->compact)  // grown on demand: room for the planes of a lone pair
       want = std::max(want, r2t::layout_single(q.width, q.height, q.max_disp, h->method,
                                                r2t::kPlanarBytes, false).total);
   }

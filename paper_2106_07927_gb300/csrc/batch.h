@@ -28,6 +28,9 @@ size_t batch_fixed_bytes(int n);
 // Returns 0, -2 when device memory is short, -3 on another CUDA error.
 int batch_reserve(BatchEngine** e, size_t need, size_t want, int n, bool planar);
 
+// Device bytes the engine holds (0 without one).
+size_t batch_bytes(const BatchEngine* e);
+
 // Base of the per-pair scratch (valid after batch_reserve).
 char* batch_scratch(BatchEngine* e);
 

@@ -222,6 +222,11 @@ int batch_reserve(BatchEngine** pe, size_t need, size_t want, int n, bool planar
   return grow_desc(e, n);
 }
 
+size_t batch_bytes(const BatchEngine* e) {
+  return e ? e->scratch_cap + (e->cap_pairs ? e->desc_bytes : 0) +
+                 (size_t)e->cap_pairs * kCountersPerGroup * sizeof(unsigned)
+           : 0;
+}
 char* batch_scratch(BatchEngine* e) { return e ? e->scratch : nullptr; }
 const char* batch_error(BatchEngine* e) { return e ? e->err : "no batch engine"; }
 

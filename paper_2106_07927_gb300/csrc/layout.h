@@ -9,15 +9,14 @@ namespace r2t {
 
 struct Layout {
   size_t cost, ct, agg, dl, dr, kr, mask, flip, dp, nst, nsv, dlf, fault, total;  // 0: not used
-  int planes;  // byte planes agg holds (the path count) instead of one volume of sums, or 0
+  int planes;  // byte planes agg holds instead of one volume of sums (method_planes), or 0
 };
 
 inline size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
 // Largest scratch a pair may take with path planes (5 or 9 B per DE instead of 3): an eighth of the
 // device's memory, and volumes below 4 GB (the plane kernels keep 32-bit offsets). 3840 x 2160 with
-// D = 256 takes 10.9 or 19.3 GB; larger pairs keep the small layout, so whatever fitted the
-// device still does.
+// D = 256 takes 10.9 or 19.3 GB; larger pairs keep the small layout.
 constexpr size_t kPlanarBytes = (size_t)32 << 30;
 
 // Cost 1 B/DE, aggregated volume 2 B/DE (4 when wide), census descriptors of both images

@@ -127,3 +127,49 @@ def test_settings_off_the_planes_take_the_values_of_the_sums():
         torch.cuda.synchronize()
         assert np.array_equal(binding.u16(out), ref), given
     st.close()
+
+
+def test_reported_sizes_cover_what_contexts_hold():
+    import torch
+    W, H, D = 500, 300, 128
+    left, right = _pair(2, W, H, D)
+    L, R = torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda()
+    out = torch.empty((H, W), dtype=torch.int16, device="cuda")
+    binding.Stereo(scenes.params(16, 16, 16, 9, 7, 10, 120, 8, 3)).close()  # the library is loaded
+    # planes (two methods), exact check, 32-bit sums, NCC
+    for p2, flags, n, planes in ((120, 3, 9, 4), (200, 7, 9, 8), (16384, 3, 9, 0),
+                                 (880, 3 | 8, 5, 0)):
+        prm = scenes.params(W, H, D, n, 7 if n == 9 else 5, 10, p2, 8, flags)
+        p = binding.params_from_dict(prm)
+        need = binding.res2tac_workspace_bytes(p)
+        torch.cuda.synchronize()
+        maps = []
+        for compact in (True, False):
+            free = torch.cuda.mem_get_info()[0]
+            st = binding.Stereo(prm, compact=compact)
+            held = binding.res2tac_context_bytes(st.handle)
+            took = free - torch.cuda.mem_get_info()[0]
+            assert abs(took - held) <= 16 << 20  # the allocator's granularity
+            if compact or not planes:
+                assert 0.9 * need < held <= need
+            else:
+                assert held >= (1 + planes) * W * H * D > need
+            maps.append(st.compute(L, R))
+            if compact and p2 <= 255 and not flags & 4:
+                pairs = [binding.res2tac_pair(L.data_ptr(), R.data_ptr(), W, out.data_ptr(), 2 * W,
+                                              W, H, D, 0)]
+                batch = binding.res2tac_batch_workspace_bytes(p, pairs)
+                for reserve in (False, True):
+                    if reserve:
+                        binding.res2tac_batch_reserve(st.handle, batch, 1)
+                    out.fill_(-1)
+                    binding.res2tac_compute_batch(st.handle, pairs,
+                                                  torch.cuda.current_stream().cuda_stream)
+                    torch.cuda.synchronize()
+                    assert torch.equal(out, maps[0])
+                    assert binding.res2tac_context_bytes(st.handle) - held <= batch + 4096
+            torch.cuda.synchronize()
+            st.close()
+        assert torch.equal(maps[0], maps[1])
+        assert np.array_equal(binding.u16(maps[0]), oracle.sgm(
+            left, right, D, prm["census_w"], prm["census_h"], 10, p2, 8, flags))
