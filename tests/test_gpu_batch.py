@@ -1,5 +1,6 @@
-"""Batch engine: uneven pairs in persistent kernels under a CUDA graph give, per pair, the same
-bits as a single-pair call and as the oracle."""
+"""Batch engine: uneven pairs give, per pair, the same bits as a single-pair call and as the oracle, on
+both of its routes: groups on path planes (P2 <= 255; one plane per two directions up to 127) and
+persistent kernels under a CUDA graph (16-bit sums, and 32-bit ones for the largest P2)."""
 import ctypes
 import itertools
 
@@ -10,6 +11,8 @@ import oracle
 from paper_2106_07927_gb300 import binding, scenes
 
 pytestmark = pytest.mark.gpu
+
+ROUTES = [120, 200, 880, 16384]  # P2
 
 
 def _run_batch(h, tensors, shapes):
@@ -77,24 +80,24 @@ def _small_batch(seed, n):
     return items
 
 
-@pytest.mark.parametrize("flags", [3, 0])
-def test_batch_matches_oracle_and_single(flags):
+@pytest.mark.parametrize("flags,p2", [(3, p) for p in ROUTES] + [(0, 120), (0, 880)])
+def test_batch_matches_oracle_and_single(flags, p2):
     import torch
     items = _small_batch(1, 10)
-    prm = scenes.params(64, 64, 64, 9, 7, 10, 120, 8, flags)
+    prm = scenes.params(64, 64, 64, 9, 7, 10, p2, 8, flags)
     ctx = binding.Stereo(prm)
     tensors = [(torch.from_numpy(L).cuda(), torch.from_numpy(R).cuda()) for L, R, _ in items]
     shapes = [s for _, _, s in items]
     outs = _run_batch(ctx.handle, tensors, shapes)
     for (L, R, (W, H, D)), got in zip(items, outs):
-        ref = oracle.sgm(L, R, D, 9, 7, 10, 120, 8, flags)
+        ref = oracle.sgm(L, R, D, 9, 7, 10, p2, 8, flags)
         assert np.array_equal(got, ref), (W, H, D)
-        single = binding.Stereo(scenes.params(W, H, D, 9, 7, 10, 120, 8, flags))
+        single = binding.Stereo(scenes.params(W, H, D, 9, 7, 10, p2, 8, flags))
         s_out = single.compute(torch.from_numpy(L).cuda(), torch.from_numpy(R).cuda())
         torch.cuda.synchronize()
         assert np.array_equal(binding.u16(s_out), got)
         single.close()
-    # replay of the captured graph with other pairs of the same layout, then a larger batch
+    # other pairs of the same layout (the persistent kernels replay their graph), then a larger batch
     items2 = _small_batch(2, 10)
     for i in range(10):
         W, H, D = shapes[i]
@@ -103,12 +106,12 @@ def test_batch_matches_oracle_and_single(flags):
     tensors2 = [(torch.from_numpy(L).cuda(), torch.from_numpy(R).cuda()) for L, R, _ in items2]
     outs2 = _run_batch(ctx.handle, tensors2, shapes)
     for (L, R, (W, H, D)), got in zip(items2, outs2):
-        assert np.array_equal(got, oracle.sgm(L, R, D, 9, 7, 10, 120, 8, flags))
+        assert np.array_equal(got, oracle.sgm(L, R, D, 9, 7, 10, p2, 8, flags))
     items3 = _small_batch(3, 17)
     tensors3 = [(torch.from_numpy(L).cuda(), torch.from_numpy(R).cuda()) for L, R, _ in items3]
     outs3 = _run_batch(ctx.handle, tensors3, [s for _, _, s in items3])
     for (L, R, (W, H, D)), got in zip(items3, outs3):
-        assert np.array_equal(got, oracle.sgm(L, R, D, 9, 7, 10, 120, 8, flags))
+        assert np.array_equal(got, oracle.sgm(L, R, D, 9, 7, 10, p2, 8, flags))
     ctx.close()
 
 
@@ -202,10 +205,12 @@ def test_batch_of_64_uneven_pairs_against_oracle():
     pool.shutdown()
 
 
-def test_every_batch_tuning_candidate_matches_oracle():
+@pytest.mark.parametrize("p2", ROUTES)
+def test_every_batch_tuning_candidate_matches_oracle(p2):
     """Every setting the batch autotuner may pick (row disparities per lane, sheared disparities
     and chains per lane, WTA tile), applied to every bucket of a small uneven batch (D from 32 to
-    256, both size classes), gives the oracle's maps; then the autotuner itself runs on that
+    256, both size classes), gives the oracle's maps (on path planes every row_dpl runs its own kernel;
+    the sheared settings have no effect there); then the autotuner itself runs on that
     batch, reports a table of valid entries and leaves maps that still match."""
     import torch
     rng = np.random.default_rng(21)
@@ -215,9 +220,9 @@ def test_every_batch_tuning_candidate_matches_oracle():
     for i, (W, H, D) in enumerate(shapes):
         L, R, _ = scenes.make_scene(("road", "nadir")[i % 2], 40 + i, W, H, D)
         items.append((L, R, (W, H, D)))
-    refs = [oracle.sgm(L, R, D, 9, 7, 10, 120, 8, 3) for L, R, (W, H, D) in items]
+    refs = [oracle.sgm(L, R, D, 9, 7, 10, p2, 8, 3) for L, R, (W, H, D) in items]
     tensors = [(torch.from_numpy(L).cuda(), torch.from_numpy(R).cuda()) for L, R, _ in items]
-    ctx = binding.Stereo(scenes.params(64, 64, 64, 9, 7, 10, 120, 8, 3))
+    ctx = binding.Stereo(scenes.params(64, 64, 64, 9, 7, 10, p2, 8, 3))
     buckets = sorted({(D, int(W * H >= (1 << 18))) for W, H, D in shapes})
     tried = 0
     for row, (sd, sc), wpx in itertools.product((2, 4, 8), ((16, 1), (16, 2)), (64, 128, 256)):
