@@ -12,9 +12,9 @@
 namespace r2t {
 
 __global__ void __launch_bounds__(256) census_kernel(Problem pb, Method mt) {
-  launch_dependents();
   __shared__ CensusSmem sm;
   census_tile_dispatch(pb, mt, blockIdx.x, sm);
+  launch_dependents();
 }
 
 __global__ void __launch_bounds__(256) cost_kernel(Problem pb, Method mt) {
@@ -35,9 +35,9 @@ __global__ void __launch_bounds__(256) cost_planar_kernel(Problem pb, Method mt)
 template <int R>
 __global__ void __launch_bounds__(256) wta_planar_kernel(Problem pb, int paths, int T) {
   wait_prerequisites();
-  launch_dependents();
   extern __shared__ __align__(16) uint8_t wsm[];
   planar_wta_tile<R>(pb, paths, blockIdx.x, wsm, T);
+  launch_dependents();
 }
 
 template <bool WIDE>
