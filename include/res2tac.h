@@ -312,8 +312,8 @@ int res2tac_set_batch_tuning(res2tac_t h, const res2tac_batch_tuning* t, int32_t
 int res2tac_get_batch_tuning(res2tac_t h, res2tac_batch_tuning* t);
 
 /* Autotuner of the batch engine: for the buckets the n pairs fall into (largest total work
- * first; each starts from the defaults) it times the whole batch (res2tac_compute_batch on stream s, median of 3 runs after one
- * warm-up) for each candidate of one setting at a time - row_dpl, then (shear_dpl, shear_cpl),
+ * first; each starts from the defaults) it times the whole batch (res2tac_compute_batch on stream s,
+ * median of 3 runs after one warm-up) for each candidate of one setting at a time - row_dpl, then (shear_dpl, shear_cpl),
  * then wta_px - keeping the fastest, and leaves the chosen table in the context, as explicit
  * settings. Candidates that run the same kernels as another one are not timed. It writes up to
  * cap entries of the buckets it tuned into table (count into *count) and the batch times before
@@ -329,7 +329,8 @@ int res2tac_last_launch_count(res2tac_t h);
 
 /* Per-stage timing. With profiling enabled, res2tac_compute records a CUDA event on the caller's
  * stream before and after each stage. res2tac_stage_times waits for the last call and writes up
- * to n durations in milliseconds: [0] census + cost (+ clearing of the aggregated volume),
+ * to n durations in milliseconds: [0] census + cost (+ clearing of the aggregated volume, without
+ * path planes),
  * [1] path aggregation, [2] WTA + right-disparity keys, [3] LR check + median. With
  * RES2TAC_EXACT_CC, [0] .. [2] add up both passes (and [0] the flip of the pair). */
 int res2tac_set_profiling(res2tac_t h, int enable);
@@ -350,8 +351,9 @@ int res2tac_stage_times(res2tac_t h, float* ms, int n);
  * 5 B per W*H*D when num_paths * (255 + p2) > 65535, 4 B more per pixel with RES2TAC_EXACT_CC,
  * 24 B more per pixel and 2 KB with RES2TAC_NCC)
  * is rejected with RES2TAC_ENOMEM and a
- * message giving both sizes. Where it fits, the array holds path planes (see res2tac_create). 640 x 480 with D = 64 fits with 16-bit sums
- * (num_paths * (255 + p2) <= 65535: about 67 MB) but not with 32-bit ones (about 106 MB).
+ * message giving both sizes. Where they fit, the array holds path planes (see res2tac_create).
+ * 640 x 480 with D = 64 fits with 16-bit sums (num_paths * (255 + p2) <= 65535: about 67 MB) but
+ * not with 32-bit ones (about 106 MB).
  * Set-up: the first call on a device looks up the array's device address (cudaGetSymbolAddress)
  * with that device current; make that first call before any stream capture.
  * Sharing: every call in the process uses the same array, which keeps the contents of the last

@@ -646,7 +646,8 @@ int res2tac_compute_batch(res2tac_t h, const res2tac_pair* pairs, int32_t n, res
       return fail(RES2TAC_EINVAL, "pair %d: bad pitch", i);
     offs[i] = total;
     total += layout_for(q.width, q.height, q.max_disp, wide).total;
-    if (planar && !h->batch_reserved && !h->compact)  // grown on demand: room for the planes of a lone pair
+    // grown on demand: room for the planes of a lone pair
+    if (planar && !h->batch_reserved && !h->compact)
       want = std::max(want, r2t::layout_single(q.width, q.height, q.max_disp, h->method,
                                                r2t::kPlanarBytes, false).total);
   }

@@ -12,9 +12,9 @@ enum {
 
 // Kernel settings of the batch for one bucket of pairs (see tune_bucket): disparities per lane of
 // the row kernel (2, 4 or 8), disparities and chains per lane of the sheared kernel (16 with 1
-// or 2 chains), pixels per WTA tile (64, 128 or 256, capped so the tile's sums take at most
-// 64 KB). The persistent sheared kernel holds every setting it may meet inlined, so its settings
-// are kept to the two that cost the most compile time to leave out.
+// or 2 chains; not on path planes), pixels per WTA tile (64, 128 or 256, capped so the tile's sums
+// take at most 64 KB, on path planes 29 KB). The persistent sheared kernel holds every setting it may
+// meet inlined, so its settings are kept to two (four doubled its compile time).
 struct BatchTune {
   signed char row_dpl, shear_dpl, shear_cpl;
   signed char automatic;  // 1: the default, which a batch on path planes may adapt to its rows

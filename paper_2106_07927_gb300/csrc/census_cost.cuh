@@ -326,7 +326,8 @@ __device__ __forceinline__ void cost_tile_planar(const Problem& pb, int item, Co
           v2 = m < h + 2 ? kCostOutside : v2;
           v3 = m < h + 3 ? kCostOutside : v3;
         }
-        if (kb + k < end) o[(kb + k) * nq] = make_uint2(pack_bytes(u0, v0, u1, v1), pack_bytes(u2, v2, u3, v3));
+        if (kb + k < end)
+          o[(kb + k) * nq] = make_uint2(pack_bytes(u0, v0, u1, v1), pack_bytes(u2, v2, u3, v3));
         // one pixel right: both windows move by one descriptor
         a3 = a2;
         a2 = a1;

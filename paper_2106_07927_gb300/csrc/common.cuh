@@ -19,7 +19,7 @@ __host__ __device__ inline int pow2ceil(int v) {
 }
 
 // Everything a kernel needs to know about one stereo pair. Volumes are [y][x][d] with the D
-// disparities of a pixel contiguous and in natural order.
+// disparities of a pixel contiguous, in natural order or (planar) in the pair order of planar.cuh.
 struct Problem {
   const uint8_t* left;
   const uint8_t* right;
@@ -29,7 +29,7 @@ struct Problem {
   int W, H, D;
   uint8_t* cost;      // [H][W][D]
   uint64_t* ct;       // [2][H][W] census descriptors of the left, then the right image
-  void* agg;          // [H][W][D], uint16 (or uint32 when wide)
+  void* agg;          // [H][W][D], uint16 (or uint32 when wide); planar: byte planes of W H D each
   uint16_t* dl;       // [H][W] winner-takes-all map
   uint16_t* dr;       // [H][W] approximate right map
   uint32_t* kr;       // [H][W] right-disparity keys S << 8 | d, reduced with atomicMin
@@ -86,10 +86,11 @@ struct Method {
 // Programmatic dependent launch (launch_dep, launch_agg): lets the next kernel of the stream start its
 // blocks once every block of this one has called it or ended / waits until the kernel before this
 // one is complete and its stores are visible. Stages of one pair call the first at their end, so the
-// next stage's launch overlaps their last blocks: 320x240, D = 64 47 -> 38 us a call, 1242x375, D =
-// 128 257 -> 249. Called at the start, the next stage's blocks take the places of this one's, and
-// the row chains sit unevenly: 317 us. Groups of a batch overlap on several streams and keep plain
-// launches (dependent ones: 1.60 instead of 1.35 ms for 64 x 320x240).
+// next stage's launch overlaps their last blocks: 320x240, D = 64, 4 paths 47.1 -> 37.6 us a call,
+// 1242x375, D = 128 256.6 -> 246.4. Called at the cost kernel's start, the row kernel's blocks take
+// the places of its blocks, and the row chains sit unevenly: 317 us. The row kernel calls it as soon
+// as its own wait is over, because the sheared kernel runs beside it. Groups of a batch overlap on
+// several streams and keep plain launches (dependent ones: 1.60 instead of 1.35 ms for 64 x 320x240).
 __device__ __forceinline__ void launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

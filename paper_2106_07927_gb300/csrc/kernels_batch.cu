@@ -566,8 +566,8 @@ int batch_run(BatchEngine* e, const Problem* probs, int n, const Method& mt, cud
 // ------------------------------------------------------------------------------- path planes
 // Batches on path planes: groups of pairs of one D, one launch per stage and group (6), no
 // descriptors in memory and no work queues. Against the persistent kernels above, which add into
-// 16-bit sums: 64 x 320x240, D = 64 1.78 -> 1.34 ms; 16 x 1242x375, D = 128 4.82 -> 3.83 ms; 16
-// uneven pairs up to 1920x1080, D = 256 11.9 -> 7.3 ms.
+// 16-bit sums: 64 x 320x240, D = 64 1.77 -> 1.30 ms; 16 x 1242x375, D = 128 4.83 -> 3.78 ms; 16
+// uneven pairs up to 1920x1080, D = 256 11.9 -> 7.4 ms.
 // Estimates (W H D) of one group: a quarter of the batch's, so that every stream has work, within these
 // bounds (a larger pair is a group of its own). Smaller groups leave the GPU to launches and to the
 // latency of the chains, larger ones the streams without work. us with groups of at least 5, 12 and

@@ -11,7 +11,8 @@ struct Tuning {
   int agg_dpl;    // disparities per lane of the row aggregation kernel (2, 4 or 8)
   int agg_warps;  // warps per aggregation block
   int wta_chunk;  // pixels per block of the WTA / right-disparity stage
-  int shear_dpl;  // disparities per lane of the sheared-column kernel (16 or 32)
+  int shear_dpl;  // disparities per lane of the sheared-column kernel (8, 16 or 32; on path planes 16,
+                  // or 8 for one chain per warp)
   int shear_cpl;  // chains per lane of the sheared-column kernel (1 or 2)
   int row_split;  // 1: one row direction per lane group, 0: both directions in one group
   int cost_mode;  // 0: population-count cost kernel, 1: tensor-core cost kernel (cost_mma_ok)
@@ -87,10 +88,11 @@ inline cudaError_t launch_agg(void (*kernel)(P...), int grid, int threads, size_
 // Pixels per tile of the selection on path planes for the setting wta_chunk / wta_px.
 int planar_tile_px(int D, int wta_px);
 // Settings the plane kernels have (blocks are always one pair of warps): 16 disparities and one chain
-// per lane of the sheared chains, or (8) one chain per warp, one row direction per lane group, costs from the
-// volume of the population-count kernel.
+// per lane of the sheared chains, or (8) one chain per warp, one row direction per lane group, costs
+// from the volume of the population-count kernel.
 inline bool planar_tuning(const Tuning& tn) {
-  return (tn.shear_dpl == 8 || tn.shear_dpl == 16) && tn.shear_cpl == 1 && tn.row_split == 1 && tn.cost_mode == 0 && tn.row_cost == 0;
+  return (tn.shear_dpl == 8 || tn.shear_dpl == 16) && tn.shear_cpl == 1 && tn.row_split == 1 &&
+         tn.cost_mode == 0 && tn.row_cost == 0;
 }
 // Persistent batch variants of the two kernels, as handles for cudaLaunchKernel. Parameters:
 // (const BatchHeader*, const GroupDesc*, const Problem*, const AggSeg* segs,
@@ -103,15 +105,17 @@ template <bool WIDE>
 const void* batch_shear_kernel_fn();
 
 // Plain single-pair pipeline: 6 kernel launches on stream s (census of both images; cost +
-// clearing of the aggregated volume; two aggregation kernels; WTA + right-disparity keys; LR
-// check + median). With the exact check (mt.flags & 4; pb.flip and pb.dp set) first a flip kernel
-// and the first five launches again on the swapped, flipped pair: 12 launches. The NCC cost
+// clearing of the aggregated volume, which path planes do not need; two aggregation kernels; WTA +
+// right-disparity keys; LR check + median). With the exact check (mt.flags & 4; pb.flip and pb.dp
+// set) first a flip kernel and the first five launches again on the swapped, flipped pair: 12
+// launches. The NCC cost
 // (mt.flags & 8) takes 3 launches instead of 2 per pass.
 // Returns the number of launches through *launches.
 // ev: NULL, or events recorded around the stages: 5 (before the cost stage, after each of the
 // four), with the exact check 8 (before the flip; after the cost, aggregation and WTA of each
 // pass; after the LR check + median).
-// fork: NULL runs the two aggregation kernels one after the other on s.
+// fork: NULL runs the two aggregation kernels one after the other on s; path planes do not use it
+// (their sheared kernel is a dependent launch beside the row kernel on s).
 cudaError_t run_pipeline(const Problem& pb, const Method& mt, const Tuning& tn, cudaStream_t s,
                          int* launches, cudaEvent_t* ev = nullptr, const Fork* fork = nullptr);
 

@@ -700,9 +700,13 @@ __device__ __forceinline__ void planar_long(const Problem& pb, const Method& mt,
 // instruction adds the number and takes the minimum of two sums; the least key has the least
 // sum and, among equal ones, the smallest d.
 // Pixels of a tile: whole blocks of 16 words along a diagonal, at most T and at most 29 KB of sums, past
-// which the SM has too little left for the L1, which holds the loads in flight. Stage us at 1281 x
-// 720 with 32, 64, 96, 128 pixels: D = 48 95, 64, -, 52; D = 64 98, 68, -, 59; D = 128 121, 101, 99, 115;
-// D = 160 146, 129, 152, -; D = 224 182, 166, 174, -; D = 256 195, 214, 220, -.
+// which the SM has too little left for the L1, which holds the loads in flight. Stage us with 32, 64,
+// 96, 128 pixels, 4 planes, 1281 x 720: D = 64 98, 68, 61, 55; D = 128 121, 100, 100, 115; D = 160 147,
+// 129, 152, 154; D = 224 182, 166, 174, 184; D = 256 195, 215, 219, -; 1920 x 1080: D = 128 260, 221,
+// 219, 234; D = 256 430, 461, 466, -; 8 planes: D = 128 430, 397, 385, 406; D = 256 794, 797, 842, -.
+// From 320 x 240 to 1920 x 1080 and 700 x 2000 the choice is within 4 % of the best of 32 .. 256 for D
+// >= 64 (within the clock's 2 us on the small ones). Below it T is the bound, and 256 pixels would
+// take 0.8 of the stage at D = 16.
 __host__ __device__ inline int planar_wta_px(int D, int T) {
   const int cap = (29500 / (4 * (D / 2 + 1))) & ~31;
   return T < cap ? T : cap;

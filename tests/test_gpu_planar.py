@@ -61,7 +61,7 @@ def test_batch_groups_and_scratch_limits(p2):
         want.append(oracle.sgm(left, right, D, 9, 7, 10, p2, 8, 3))
     params = binding.params_from_dict(prm)
     one = binding.res2tac_batch_workspace_bytes(params, pairs[-1:])
-    # grown on demand; reserved for the batch; reserved for less than the large pair's planes
+    # grown on demand; reserved for the batch; reserved for the large pair alone
     for reserve, batch in ((0, pairs), (binding.res2tac_batch_workspace_bytes(params, pairs), pairs),
                            (one, pairs[-1:])):
         ctx = binding.Stereo(prm)
