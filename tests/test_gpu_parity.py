@@ -401,12 +401,18 @@ def test_maximum_width_and_height(W, H):
     _assert_same(left, right, scenes.params(W, H, 64, 5, 5, 10, 120, 8, 3))
 
 
-def test_3840x2160_d256_sampled_sums():
-    # the largest pair of the serving workload: the aggregated sums at sampled pixels (corners,
-    # borders, interior) from the oracle's walk along the 8 path lines through each of them
+# the largest pair of the serving workload, and the most estimates path planes take (offsets of up to
+# 2^32): the aggregated sums at sampled pixels (corners, borders, interior) from the oracle's walk
+# along the 8 path lines through each of them
+@pytest.mark.parametrize("W,H", [(3840, 2160), (8192, 2040)])
+def test_large_pairs_d256_sampled_sums(W, H):
     import torch
-    W, H, D = 3840, 2160, 256
-    left, right, _ = scenes.make_scene("road", 5, W, H, D)
+    D = 256
+    if W > 4000:
+        left = np.random.default_rng(5).integers(0, 256, (H, W)).astype(np.uint8)
+        right = np.roll(left, -70, axis=1)
+    else:
+        left, right, _ = scenes.make_scene("road", 5, W, H, D)
     prm = scenes.params(W, H, D, 9, 7, 10, 120, 8, 3)
     st = binding.Stereo(prm)
     st.compute(torch.from_numpy(left).cuda(), torch.from_numpy(right).cuda())
