@@ -63,13 +63,14 @@ def test_captured_batch_keeps_its_scratch(p2):
     pairs = descriptors(images, outs, shapes)
     batch = lambda ps: binding.res2tac_compute_batch(ctx.handle, ps,
                                                      torch.cuda.current_stream().cuda_stream)
-    # an earlier batch with one pair twice as high sized the scratch
+    # an earlier batch sized the scratch
     tall = [(300, 100, 64)] * 12 + [(300, 200, 64)] * 3
     ims = [[torch.from_numpy(a).cuda() for a in _pair(40 + i, *s)] for i, s in enumerate(tall)]
     maps = [torch.empty((H, W), dtype=torch.int16, device="cuda") for W, H, D in tall]
     batch(descriptors(ims, maps, tall))
     g = _captured(torch, lambda: batch(pairs))
-    # a lone pair whose sums fit the scratch and whose planes (5 or 9 bytes per estimate) do not
+    # a lone pair whose sums fit what that batch needs and whose planes (5 or 9 bytes per estimate) do
+    # not
     prm = binding.params_from_dict(scenes.params(64, 64, 64, 9, 7, 10, p2, 8, 3))
     held = binding.res2tac_batch_workspace_bytes(prm, descriptors(ims, maps, tall))
     W, D = 640, 128
@@ -77,11 +78,11 @@ def test_captured_batch_keeps_its_scratch(p2):
     assert H * W * (3 * D + 25) < 0.8 * held
     lone = [torch.from_numpy(a).cuda() for a in _pair(77, W, H, D)]
     lone_out = torch.empty((H, W), dtype=torch.int16, device="cuda")
-    torch.cuda.synchronize()
-    before = torch.cuda.mem_get_info()[0]
+    before = binding.res2tac_context_bytes(ctx.handle)
     batch(descriptors([lone], [lone_out], [(W, H, D)]))
     torch.cuda.synchronize()
-    assert torch.cuda.mem_get_info()[0] == before  # the scratch stayed where the graph has it
+    # the scratch stayed where the graph has it
+    assert binding.res2tac_context_bytes(ctx.handle) == before
     for i, s in enumerate(shapes):
         left, right = _pair(100 + i, *s)
         images[i][0].copy_(torch.from_numpy(left))
@@ -96,7 +97,7 @@ def test_captured_batch_keeps_its_scratch(p2):
     want = single.compute(*lone)
     torch.cuda.synchronize()
     assert torch.equal(want, lone_out)
-    # a call under capture whose planes do not fit allocates nothing either
+    # a call under capture allocates nothing either
     g2 = torch.cuda.CUDAGraph()
     with torch.cuda.graph(g2):
         batch(descriptors([lone], [lone_out], [(W, H, D)]))
